@@ -159,12 +159,12 @@ int tvlbm_set_scheme(tvlbm_ctx *ctx, int scheme, double tau_g);
 int tvlbm_set_fv_pressure_scaling(tvlbm_ctx *ctx, int enable);
 
 /* Finite-volume scheme: one fused kernel per step (fused = 1, default) or two (fused = 0).  The
- * fused kernel computes the collision term of Eq. OMEGAFVLB for a block of cells in shared memory
- * and updates the block's inner cells from it (Eq. FVLB): Q values read and Q written per cell
- * update.  The two-kernel form stores the collision term of every cell in the buffer
- * tvlbm_set_scheme allocates and reads it back in the update (5 Q values per cell update).  Both
- * run the same arithmetic and give the same populations bit for bit.  May be called at any time;
- * takes effect at the next step.  Errors: EINVAL (null context). */
+ * fused kernel computes the collision term of Eq. OMEGAFVLB in registers and updates the cells from
+ * it (Eq. FVLB): Q values read and Q written per cell update.  The two-kernel form stores the
+ * collision term of every cell in the buffer tvlbm_set_scheme allocates and reads it back in the
+ * update (5 Q values per cell update); FP64 storage, bound by its arithmetic, always runs it.  Both
+ * give the same populations bit for bit.  May be called at any time; takes effect at the next step.
+ * Errors: EINVAL (null context). */
 int tvlbm_set_fv_fused(tvlbm_ctx *ctx, int fused);
 
 /* Finite-volume scheme on a channel (a context created with TVLBM_BC_WALLS): the first and

@@ -416,7 +416,7 @@ int tvlbm_destroy(tvlbm_ctx* c) {
     for (int k = 0; k < 2; ++k)
         if (c->cl_graph[k]) cudaGraphExecDestroy(c->cl_graph[k]);
     if (c->fv_omega) cudaFree(c->fv_omega);
-    if (c->fv_dy) cudaFree(c->fv_dy);
+    if (c->fv_ysc) cudaFree(c->fv_ysc);
     if (c->fv_wall_eq) cudaFree(c->fv_wall_eq);
     if (c->mesh_mem) cudaFree(c->mesh_mem);
     if (c->ref_mem) cudaFree(c->ref_mem);

@@ -243,6 +243,7 @@ void fill_kparams(KParams& p, const Rule& r, int N, double dt, double tau, doubl
         shift_of(r.x[i], dt, &sh, &a);
         p.sh[i] = sh;
         p.xd[i] = r.x[i];
+        p.x2d[i] = r.x[i] * r.x[i];
         p.xf[i] = (float)r.x[i];
         p.x2f[i] = p.xf[i] * p.xf[i];
         p.wd[i] = r.w[i];

@@ -64,6 +64,7 @@ struct KParams {
     // axes (tensor-product set, dx = dy).
     float xf[kMaxN1], wf[kMaxN1], af[kMaxN1];
     double xd[kMaxN1], wd[kMaxN1], ad[kMaxN1];
+    double x2d[kMaxN1];  // xd * xd
     float Ef[kMaxN1][kMaxN1];
     double Ed[kMaxN1][kMaxN1];
     float x2f[kMaxN1];   // float(xf * xf)
@@ -154,7 +155,7 @@ __host__ __device__ __forceinline__ Geom geom_of(const KParams& p) {
 }
 
 template <class R> __device__ __forceinline__ R kx2(const KParams& p, int i) {
-    if constexpr (std::is_same<R, double>::value) return p.xd[i] * p.xd[i]; else return p.x2f[i];
+    if constexpr (std::is_same<R, double>::value) return p.x2d[i]; else return p.x2f[i];
 }
 template <class R> __device__ __forceinline__ R kw(const KParams& p, int i) {
     if constexpr (std::is_same<R, double>::value) return p.wd[i]; else return p.wf[i];
@@ -370,10 +371,10 @@ __device__ __forceinline__ void cell_collide(R (&s)[N1 * N1], const KParams& p, 
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// Launch a kernel with programmatic stream serialization (see pdl_wait).
+// Launch a kernel, with programmatic stream serialization (see pdl_wait) or without.
 template <class... KArgs, class... Args>
-inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                              Args&&... args) {
+inline cudaError_t launch_as(bool pdl, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                             Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -383,8 +384,13 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+template <class... KArgs, class... Args>
+inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                              Args&&... args) {
+    return launch_as(true, kernel, grid, block, smem, s, std::forward<Args>(args)...);
 }
 
 // Explicit global-space stores and loads: the population buffers are always global memory, and
