@@ -1,15 +1,14 @@
-// The closure network on Blackwell tensor cores: every matrix product of inference and training
-// is one tcgen05 GEMM kernel, D[rows x BN] = A[rows x K] * B[BN x K]^T with BF16 operands in
-// K-major layout (TMA 2-D loads, 128-byte swizzle, a STAGES-deep ring of shared-memory stages),
-// the FP32 accumulator in TMEM, and an epilogue that reads TMEM row by row (thread = row) and
-// fuses bias, GELU, its derivative, the loss, transposed copies and bias gradients.
+// The closure network on Blackwell tensor cores: inference and training each run as one kernel per
+// 128-row tile in which every matrix product is a chain of tcgen05 MMAs (BF16 operands in
+// 128-byte-swizzled shared memory, FP32 accumulators in TMEM) and the epilogues between them read
+// TMEM row by row and fuse bias, GELU, its derivative, the loss and the bias gradients.
 //
 // Forward:  Z1 = X W1^T + b1, H1 = g(Z1);  Z2 = H1 W2^T + b2, H2 = g(Z2);  Y = H2 W3^T + b3.
 // Backward (L = mean (Y - Y*)^2):  dY = 2 (Y - Y*) / (rows 12);  dZ2 = (dY W3) o g'(Z2);
-//   dZ1 = (dZ2 W2) o g'(Z1);  dW3 = dY^T H2, dW2 = dZ2^T H1, dW1 = dZ1^T X (split over rows,
-//   partial sums reduced in a fixed order);  db = column sums (atomics).
-// Every operand a later product needs transposed is written transposed by the epilogue that
-// produces it, so that all products keep K-major operands.
+//   dZ1 = (dZ2 W2) o g'(Z1);  dW3 = dY^T H2, dW2 = dZ2^T H1, dW1 = dZ1^T X (accumulated in TMEM
+//   over a CTA's tiles, the CTAs' sums reduced in a fixed order);  db = column sums.
+// No operand is ever transposed in memory: a tile stored with rows of 64 entries is a K-major
+// operand where the product contracts its columns and an MN-major one where it contracts its rows.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -24,6 +23,7 @@
 #include "tvlbm.h"
 #include "tvlbm_closure.h"
 #include "tvlbm_host.h"
+#include "tvlbm_kernels.cuh"
 #include "tvlbm_mlp.h"
 #include "tvlbm_tc.cuh"
 
@@ -32,13 +32,12 @@ using namespace tvlbm::tc;
 
 namespace {
 
-constexpr int BM = 128, BK = 64;
+constexpr int BM = 128, BK = 64;  // rows of a tile, columns of a 128-byte-swizzled chunk
 constexpr int NIN = TVLBM_MLP_IN, NINP = TVLBM_MLP_IN_PAD, NH = TVLBM_MLP_HIDDEN, NOUT = TVLBM_MLP_OUT,
               NOUTP = TVLBM_MLP_OUT_PAD;
 constexpr int OFF_W1 = 0, OFF_B1 = OFF_W1 + NH * NIN, OFF_W2 = OFF_B1 + NH, OFF_B2 = OFF_W2 + NH * NH,
               OFF_W3 = OFF_B2 + NH, OFF_B3 = OFF_W3 + NOUT * NH, NPARAM = OFF_B3 + NOUT;
 static_assert(NPARAM == TVLBM_MLP_PARAMS, "parameter count");
-constexpr int kMaxSplits = 128;
 
 using bf16 = __nv_bfloat16;
 
@@ -80,6 +79,26 @@ __device__ __forceinline__ float2 gelu2_f(float2 z) {
     const float2 er = make_float2(copysignf(r.x, x.x), copysignf(r.y, x.y));
     return __fmul2_rn(__fmul2_rn(make_float2(0.5f, 0.5f), z), __fadd2_rn(make_float2(1.0f, 1.0f), er));
 }
+// GELU and its derivative of a pair, erf and exponential shared: per lane the operations of gelu_f
+// and gelu_grad_f.
+__device__ __forceinline__ float2 gelu2_both(float2 z, float2& dg) {
+    const float2 x = __fmul2_rn(z, make_float2(0.70710678118654752f, 0.70710678118654752f));
+    const float2 ax = make_float2(fabsf(x.x), fabsf(x.y));
+    const float2 d = __ffma2_rn(make_float2(0.3275911f, 0.3275911f), ax, make_float2(1.0f, 1.0f));
+    const float2 t = make_float2(__fdividef(1.0f, d.x), __fdividef(1.0f, d.y));
+    float2 q = __ffma2_rn(t, make_float2(1.061405429f, 1.061405429f), make_float2(-1.453152027f, -1.453152027f));
+    q = __ffma2_rn(t, q, make_float2(1.421413741f, 1.421413741f));
+    q = __ffma2_rn(t, q, make_float2(-0.284496736f, -0.284496736f));
+    q = __ffma2_rn(t, q, make_float2(0.254829592f, 0.254829592f));
+    const float2 poly = __fmul2_rn(t, q);
+    const float2 sq = __fmul2_rn(make_float2(-ax.x, -ax.y), ax);
+    const float2 e2 = make_float2(__expf(sq.x), __expf(sq.y));
+    const float2 r = __ffma2_rn(make_float2(-poly.x, -poly.y), e2, make_float2(1.0f, 1.0f));
+    const float2 er1 = __fadd2_rn(make_float2(1.0f, 1.0f), make_float2(copysignf(r.x, x.x), copysignf(r.y, x.y)));
+    const float2 half = make_float2(0.5f, 0.5f);
+    dg = __ffma2_rn(__fmul2_rn(z, make_float2(0.39894228040143268f, 0.39894228040143268f)), e2, __fmul2_rn(half, er1));
+    return __fmul2_rn(__fmul2_rn(half, z), er1);
+}
 __device__ __forceinline__ float gelu_grad_f(float z) {
     float e2;
     const float er = erf_as(z * 0.70710678118654752f, e2);
@@ -108,240 +127,6 @@ __device__ __forceinline__ float warp_sum_f(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
-}
-
-// ---- epilogues: called by every thread with its row and 16 consecutive accumulator columns ----
-
-// Hidden layer: h = g(z + b) to H[row][col] (and H^T[col][row]); g'(z + b) to G[row][col].
-struct EpiHidden {
-    const float* bias;
-    bf16* H;   // [rows][128] or null
-    bf16* HT;  // [128][ldt] or null
-    bf16* G;   // [rows][128] or null
-    int ldt;
-    __device__ void operator()(int row, int c0, const float (&v)[16], int /*lane*/) const {
-        alignas(16) bf16 h[16], gg[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            const float z = v[k] + bias[c0 + k];
-            h[k] = __float2bfloat16_rn(gelu_f(z));
-            gg[k] = __float2bfloat16_rn(gelu_grad_f(z));
-        }
-        if (H) {
-            uint4* d = reinterpret_cast<uint4*>(H + (size_t)row * NH + c0);
-            d[0] = reinterpret_cast<const uint4*>(h)[0];
-            d[1] = reinterpret_cast<const uint4*>(h)[1];
-        }
-        if (G) {
-            uint4* d = reinterpret_cast<uint4*>(G + (size_t)row * NH + c0);
-            d[0] = reinterpret_cast<const uint4*>(gg)[0];
-            d[1] = reinterpret_cast<const uint4*>(gg)[1];
-        }
-        if (HT) {
-#pragma unroll
-            for (int k = 0; k < 16; ++k) HT[(size_t)(c0 + k) * ldt + row] = h[k];
-        }
-    }
-};
-
-// Output layer: y = z + b3 to Y (FP32 [rows][16]); with targets, dY = scale (y - y*) to
-// dY[row][0..15] (BF16, row length 64) and dY^T[col][row], the loss sum and db3.
-struct EpiOut {
-    const float* bias;
-    float* Y;            // [rows][16] or null
-    const float* ystar;  // [rows][16] or null (inference)
-    bf16* dY;            // [rows][64]
-    bf16* dYT;           // [16][ldt]
-    double* loss;
-    float* db;  // gradient of b3 (12)
-    float scale;
-    int ldt;
-    __device__ void operator()(int row, int c0, const float (&v)[16], int lane) const {
-        float y[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) y[k] = k < NOUT ? v[k] + bias[k] : 0.0f;
-        if (Y) {
-            float4* d = reinterpret_cast<float4*>(Y + (size_t)row * NOUTP);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) d[q] = make_float4(y[4 * q], y[4 * q + 1], y[4 * q + 2], y[4 * q + 3]);
-        }
-        if (!ystar) return;
-        (void)c0;
-        float sq = 0.0f;
-        alignas(16) bf16 g[16];
-        float gf[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            const float d = k < NOUT ? y[k] - ystar[(size_t)row * NOUTP + k] : 0.0f;
-            sq = fmaf(d, d, sq);
-            gf[k] = scale * d;
-            g[k] = __float2bfloat16_rn(gf[k]);
-        }
-        uint4* d = reinterpret_cast<uint4*>(dY + (size_t)row * NINP);
-        d[0] = reinterpret_cast<const uint4*>(g)[0];
-        d[1] = reinterpret_cast<const uint4*>(g)[1];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) dYT[(size_t)k * ldt + row] = g[k];
-        const float s = warp_sum_f(sq);
-        if (lane == 0) atomicAdd(loss, (double)s);
-#pragma unroll
-        for (int k = 0; k < NOUT; ++k) {
-            const float t = warp_sum_f(gf[k]);
-            if (lane == 0) atomicAdd(db + k, t);
-        }
-    }
-};
-
-// Back through a GELU: dz = acc o G to dZ[row][col] (optional) and dZ^T[col][row]; db += dz.
-struct EpiBack {
-    const bf16* G;  // [rows][128]
-    bf16* dZ;       // [rows][128] or null
-    bf16* dZT;      // [128][ldt]
-    float* db;      // [128]
-    int ldt;
-    __device__ void operator()(int row, int c0, const float (&v)[16], int lane) const {
-        alignas(16) bf16 gb[16], z[16];
-        const uint4* gs = reinterpret_cast<const uint4*>(G + (size_t)row * NH + c0);
-        reinterpret_cast<uint4*>(gb)[0] = gs[0];
-        reinterpret_cast<uint4*>(gb)[1] = gs[1];
-        float dz[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            dz[k] = v[k] * __bfloat162float(gb[k]);
-            z[k] = __float2bfloat16_rn(dz[k]);
-        }
-        if (dZ) {
-            uint4* d = reinterpret_cast<uint4*>(dZ + (size_t)row * NH + c0);
-            d[0] = reinterpret_cast<const uint4*>(z)[0];
-            d[1] = reinterpret_cast<const uint4*>(z)[1];
-        }
-#pragma unroll
-        for (int k = 0; k < 16; ++k) dZT[(size_t)(c0 + k) * ldt + row] = z[k];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            const float t = warp_sum_f(dz[k]);
-            if (lane == 0) atomicAdd(db + c0 + k, t);
-        }
-    }
-};
-
-// Split-K partial sums: part[split][row][col] (row < 128, ld = BN).
-struct EpiPartial {
-    float* part;
-    int ld;
-    __device__ void operator()(int row, int c0, const float (&v)[16], int /*lane*/) const {
-        float* d = part + ((size_t)blockIdx.y * BM + row) * ld + c0;
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            reinterpret_cast<float4*>(d)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-    }
-};
-
-// ---- the GEMM kernel ---------------------------------------------------------------------------
-template <int BN, int STAGES>
-struct GemmCfg {
-    static constexpr int A_BYTES = BM * BK * 2;  // 16 KB
-    static constexpr int B_BYTES = BN * BK * 2;
-    static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;  // multiple of 1024
-    static constexpr int SMEM = STAGES * STAGE_BYTES + 1024;
-    static constexpr uint32_t TMEM_COLS = BN < 32 ? 32 : BN;
-    static_assert(STAGE_BYTES % 1024 == 0, "stages must keep 1024-byte alignment");
-    static_assert(BN % 16 == 0 && BN >= 16 && BN <= 256, "N of a kind::f16 MMA with M = 128");
-};
-
-// CTA (blockIdx.x, blockIdx.y): rows [128 x, 128 x + 128), K chunks [y cps, min(kchunks, (y+1) cps)).
-// Thread 0 loads stages and issues the MMAs; all 128 threads then drain TMEM through the epilogue
-// (warp w owns TMEM lanes, i.e. rows, 32 w .. 32 w + 31).
-template <int BN, int STAGES, class Epi>
-__global__ void __launch_bounds__(128) gemm_kernel(const __grid_constant__ CUtensorMap ma,
-                                                   const __grid_constant__ CUtensorMap mb, int kchunks, int cps, Epi epi,
-                                                   int* status) {
-    using Cfg = GemmCfg<BN, STAGES>;
-    extern __shared__ unsigned char smem_raw[];
-    unsigned char* base = smem_raw + ((1024u - (saddr(smem_raw) & 1023u)) & 1023u);
-    __shared__ uint64_t full[STAGES], empty[STAGES], done;
-    __shared__ uint32_t tmem_slot;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.x * BM;
-    const int k0 = blockIdx.y * cps;
-    const int nk = min(kchunks, k0 + cps) - k0;  // >= 1 (host grid)
-
-    if (tid == 0) {
-#pragma unroll
-        for (int s = 0; s < STAGES; ++s) {
-            bar_init(&full[s], 1);
-            bar_init(&empty[s], 1);
-        }
-        bar_init(&done, 1);
-        bar_init_fence();
-    }
-    if (warp == 0) tmem_alloc(&tmem_slot, Cfg::TMEM_COLS);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = tmem_slot;
-
-    bool ok = true;
-    if (tid == 0) {
-        const uint32_t idesc = idesc_bf16_f32(BM, BN);
-        auto load = [&](int c) {
-            const int s = c % STAGES;
-            unsigned char* a = base + s * Cfg::STAGE_BYTES;
-            bar_expect_tx(&full[s], (uint32_t)Cfg::STAGE_BYTES);
-            tma_load_2d(a, &ma, &full[s], (k0 + c) * BK, m0);
-            tma_load_2d(a + Cfg::A_BYTES, &mb, &full[s], (k0 + c) * BK, 0);
-        };
-        const int pre = nk < STAGES ? nk : STAGES;
-        for (int c = 0; c < pre; ++c) load(c);
-        int issued = pre;
-        for (int c = 0; c < nk; ++c) {
-            const int s = c % STAGES;
-            const uint32_t par = (uint32_t)((c / STAGES) & 1);
-            if (!bar_wait(&full[s], par)) {
-                ok = false;
-                break;
-            }
-            tc_fence_after();
-            const uint32_t a = saddr(base + s * Cfg::STAGE_BYTES);
-            const uint32_t b = a + Cfg::A_BYTES;
-#pragma unroll
-            for (int kk = 0; kk < BK / 16; ++kk)
-                mma_bf16(tmem, sw128_desc(a + kk * 32), sw128_desc(b + kk * 32), idesc, c > 0 || kk > 0);
-            mma_commit(&empty[s]);
-            if (c + STAGES < nk) {
-                if (!bar_wait(&empty[s], par)) {  // the MMAs reading stage s are done
-                    ok = false;
-                    break;
-                }
-                load(c + STAGES);
-                ++issued;
-            }
-        }
-        mma_commit(&done);
-        if (!ok) {
-            // let every issued load land before the CTA exits (bounded)
-            for (int c = 0; c < issued; ++c) bar_wait(&full[c % STAGES], (uint32_t)((c / STAGES) & 1));
-        }
-    }
-    const bool ready = bar_wait(&done, 0);
-    const bool all = __syncthreads_and(ready && ok) != 0;
-    tc_fence_after();
-    if (all) {
-        const int row = m0 + warp * 32 + lane;
-        const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);
-#pragma unroll 1
-        for (int c0 = 0; c0 < BN; c0 += 16) {
-            float v[16];
-            __syncwarp();
-            tmem_ld16(taddr + (uint32_t)c0, v);
-            epi(row, c0, v, lane);
-        }
-    } else if (tid == 0 && status) {
-        atomicOr(status, 1);
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_free(tmem, Cfg::TMEM_COLS);
 }
 
 // ---- fused inference: the three layers of one 128-row tile in one CTA ---------------------------
@@ -564,69 +349,373 @@ __global__ void __launch_bounds__(kFusedThreads) mlp_fused_forward_kernel(const 
     if (warp == 0) tmem_free(tmem, FusedCfg::TMEM_COLS);
 }
 
+// Sums over the 32 lanes of 32 values a lane: lane c returns the sum of every lane's v[c] (halving
+// exchange: 31 shuffles where 32 separate warp sums take 160).  v is overwritten.
+__device__ __forceinline__ float column_sums32(float (&v)[32], int lane) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int k = 0; k < o; ++k) {
+            const float send = up ? v[k] : v[k + o], keep = up ? v[k + o] : v[k];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+    return v[0];
+}
+
+// ---- training: forward and backward of the 128-row tiles of a CTA ---------------------------------
+// Shared memory: the weights (loaded once), the input tile, H1 and H2 (later overwritten by dZ1 and
+// dZ2, once the products that read them are done) and dY, all as 64-column chunks with 128-byte
+// rows.  TMEM (512 columns): the three weight gradients, accumulated over the CTA's tiles, Y, and
+// two 128-column work areas.  g'(Z) stays in registers between the passes (BF16, 16 per layer).
+// The products are tiny (0.14 MFLOP a row), so the chain of epilogues bounds it: 18 us for a tile, and
+// one CTA per SM runs up to 152 tiles in that time.  A batch of 4096 rows takes 28 us (with the
+// gradient reduction and Adam) where thirteen kernels, one product each with its operands and their
+// transposes through memory, took 155 us.
+struct TrainCfg {
+    static constexpr int X_OFF = 0, W1_OFF = 16384, W2_OFF = 32768, W3_OFF = 65536, H1_OFF = 69632, H2_OFF = 102400,
+                         DY_OFF = 135168;
+    static constexpr int BYTES = DY_OFF + 16384;  // 148 KB
+    static constexpr int SMEM = BYTES + 1024;
+    static constexpr uint32_t TX_W = 16384 + 32768 + 4096, TX_X = 16384;
+    static constexpr uint32_t T_DW2 = 0, T_DW1 = 128, T_DW3 = 192, T_Y = 208, T_A = 256, T_B = 384;
+    // a CTA's partial sums, floats: dW1 [128][64], dW2 [128][128], dW3 [16][128], then the bias
+    // gradients of the four 32-row groups: db1 [4][128], db2 [4][128], db3 [4][16]
+    static constexpr int P_W1 = 0, P_W2 = P_W1 + NH * NINP, P_W3 = P_W2 + NH * NH, P_B1 = P_W3 + NOUTP * NH,
+                         P_B2 = P_B1 + 4 * NH, P_B3 = P_B2 + 4 * NH, P_TOTAL = P_B3 + 4 * NOUTP;
+};
+
+// K = 16 slices kk of D (+)= A B^T over `steps` slices, operand starts ad / bd advancing by as / bs
+// descriptor units (16 bytes) per slice.
+__device__ __forceinline__ void mma_chain(uint32_t d, uint64_t ad, uint64_t bd, uint32_t as, uint32_t bs, int steps,
+                                          uint32_t idesc, bool accumulate) {
+#pragma unroll 8
+    for (int k = 0; k < steps; ++k) mma_bf16(d, ad + (uint64_t)k * as, bd + (uint64_t)k * bs, idesc, accumulate || k > 0);
+}
+
+__global__ void __launch_bounds__(kFusedThreads, 1) mlp_train_kernel(const __grid_constant__ CUtensorMap mx,
+                                                                     const __grid_constant__ CUtensorMap mw1,
+                                                                     const __grid_constant__ CUtensorMap mw2,
+                                                                     const __grid_constant__ CUtensorMap mw3,
+                                                                     const float* __restrict__ theta,
+                                                                     const float* __restrict__ ystar, int tiles, float scale,
+                                                                     float* __restrict__ part, double* __restrict__ loss_part,
+                                                                     int* status) {
+    using Cfg = TrainCfg;
+    static_assert(kFusedGroups == 4, "32 columns per thread and hidden layer");
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* base = smem_raw + ((1024u - (saddr(smem_raw) & 1023u)) & 1023u);
+    __shared__ uint64_t w_bar, x_bar, mma_bar;
+    __shared__ __align__(16) float bias[2 * NH + NOUTP];
+    __shared__ uint32_t tmem_slot;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    pdl_launch_dependents();
+    if (tid == 0) {
+        bar_init(&w_bar, 1);
+        bar_init(&x_bar, 1);
+        bar_init(&mma_bar, 1);
+        bar_init_fence();
+    }
+    if (warp == 0) tmem_alloc(&tmem_slot, 512);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    pdl_wait();  // the weights (and the partial sums' readers) of the kernels before this one
+    const uint32_t tmem = tmem_slot;
+    unsigned char *xs = base + Cfg::X_OFF, *w1 = base + Cfg::W1_OFF, *w2 = base + Cfg::W2_OFF, *w3 = base + Cfg::W3_OFF,
+                  *h1 = base + Cfg::H1_OFF, *h2 = base + Cfg::H2_OFF, *dys = base + Cfg::DY_OFF;
+    const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    const int r = (warp & 3) * 32 + lane;  // this thread's row of the tile (= its TMEM lane)
+    const int cbeg = (warp >> 2) * 32;     // its 32 columns of a hidden layer
+    // the biases, read past the L1 cache (an earlier kernel on the stream may still have been writing
+    // them when this one was launched)
+    if (tid < NH) bias[tid] = __ldcg(theta + OFF_B1 + tid);
+    else if (tid < 2 * NH) bias[tid] = __ldcg(theta + OFF_B2 + tid - NH);
+    else if (tid < 2 * NH + NOUTP) bias[tid] = tid < 2 * NH + NOUT ? __ldcg(theta + OFF_B3 + tid - 2 * NH) : 0.0f;
+    const float *b1 = bias + cbeg, *b2 = bias + NH + cbeg, *b3 = bias + 2 * NH;
+
+    if (tid == 0) {
+        bar_expect_tx(&w_bar, Cfg::TX_W);
+        tma_load_2d(w1, &mw1, &w_bar, 0, 0);
+        tma_load_2d(w2, &mw2, &w_bar, 0, 0);
+        tma_load_2d(w2 + 16384, &mw2, &w_bar, BK, 0);
+        tma_load_2d(w3, &mw3, &w_bar, 0, 0);
+        tma_load_2d(w3 + 2048, &mw3, &w_bar, BK, 0);
+        bar_expect_tx(&x_bar, Cfg::TX_X);
+        tma_load_2d(xs, &mx, &x_bar, 0, (int)blockIdx.x * BM);
+    }
+    uint32_t ph = 0;  // phase of mma_bar
+    bool ok = true;
+    // every thread waits for the products committed last; the MMAs' reads of shared memory are done too
+    auto products_done = [&]() {
+        ok = __syncthreads_and(ok && bar_wait(&mma_bar, ph)) != 0;
+        ph ^= 1;
+        tc_fence_after();
+    };
+    // generic writes of this thread -> MMA operands
+    auto operands_ready = [&]() {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+    };
+    const uint32_t kk = idesc_bf16_f32(BM, NH), kk16 = idesc_bf16_f32(BM, NOUTP);
+    constexpr uint32_t A_MN = 1u << 15, B_MN = 1u << 16;
+    float db1 = 0.0f, db2 = 0.0f, db3 = 0.0f;  // column sums of this warp's rows: column cbeg + lane (db3: lane)
+    double loss = 0.0;
+    bool first = true;
+
+#pragma unroll 1
+    for (int tile = blockIdx.x; ok && tile < tiles; tile += gridDim.x, first = false) {
+        const int m0 = tile * BM;
+        const uint32_t xph = (uint32_t)((tile - (int)blockIdx.x) / (int)gridDim.x) & 1u;
+        float4 ys[3];
+        if (warp < 4) {  // the targets, long before they are needed
+            const float4* q = reinterpret_cast<const float4*>(ystar + (size_t)(m0 + r) * NOUTP);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) ys[k] = __ldg(q + k);
+        }
+        if (tid == 0) {
+            ok = (!first || bar_wait(&w_bar, 0)) && bar_wait(&x_bar, xph);
+            tc_fence_after();
+            if (ok) mma_chain(tmem + Cfg::T_A, sw128_desc(saddr(xs)), sw128_desc(saddr(w1)), 2, 2, BK / 16, kk, false);
+            mma_commit(&mma_bar);
+        }
+        products_done();
+        uint32_t g1[16], g2[16];  // g'(Z1), g'(Z2) of this thread's columns, BF16 pairs
+        // H = g(Z + b) into h, g'(Z + b) into gp
+        auto hidden = [&](uint32_t t0, const float* b, unsigned char* h, uint32_t (&gp)[16]) {
+#pragma unroll
+            for (int c = 0; c < 32; c += 16) {
+                float v[16];
+                __syncwarp();
+                tmem_ld16(taddr + t0 + (uint32_t)(cbeg + c), v);
+#pragma unroll
+                for (int k = 0; k < 16; k += 2) {
+                    float2 dg;
+                    const float2 g = gelu2_both(
+                        __fadd2_rn(make_float2(v[k], v[k + 1]), *reinterpret_cast<const float2*>(b + c + k)), dg);
+                    v[k] = g.x;
+                    v[k + 1] = g.y;
+                    const __nv_bfloat162 d2 = __floats2bfloat162_rn(dg.x, dg.y);
+                    gp[(c + k) / 2] = *reinterpret_cast<const uint32_t*>(&d2);
+                }
+                store_h_sw128(h, r, cbeg + c, v);
+            }
+        };
+        if (ok) hidden(Cfg::T_A, b1, h1, g1);
+        operands_ready();
+        if (tid == 0) {
+            if (ok)
+#pragma unroll
+                for (int kc = 0; kc < 2; ++kc)
+                    mma_chain(tmem + Cfg::T_B, sw128_desc(saddr(h1) + kc * 16384), sw128_desc(saddr(w2) + kc * 16384), 2, 2,
+                              BK / 16, kk, kc > 0);
+            mma_commit(&mma_bar);
+        }
+        products_done();
+        if (ok) hidden(Cfg::T_B, b2, h2, g2);
+        operands_ready();
+        if (tid == 0) {
+            if (ok)
+#pragma unroll
+                for (int kc = 0; kc < 2; ++kc)
+                    mma_chain(tmem + Cfg::T_Y, sw128_desc(saddr(h2) + kc * 16384), sw128_desc(saddr(w3) + kc * 2048), 2, 2,
+                              BK / 16, kk16, kc > 0);
+            mma_commit(&mma_bar);
+        }
+        products_done();
+        if (ok && warp < 4) {  // the loss, dY (BF16, columns 12 .. 15 zero), db3
+            float v[32];
+            {
+                float y[16];
+                __syncwarp();
+                tmem_ld16(taddr + Cfg::T_Y, y);
+                const float* t = reinterpret_cast<const float*>(ys);
+                float sq = 0.0f;
+#pragma unroll
+                for (int k = 0; k < 16; ++k) {
+                    const float d = k < NOUT ? (y[k] + b3[k]) - t[k < NOUT ? k : 0] : 0.0f;
+                    sq = fmaf(d, d, sq);
+                    y[k] = scale * d;
+                    v[k] = y[k];
+                    v[k + 16] = 0.0f;
+                }
+                store_h_sw128(dys, r, 0, y);
+                const float s = warp_sum_f(sq);
+                loss += (double)s;
+            }
+            db3 += column_sums32(v, lane);
+        }
+        operands_ready();
+        if (tid == 0) {
+            if (ok) {
+                // dH2 = dY W3 (contracts the 16 outputs), dW3^T += H2^T dY (contracts the rows)
+                mma_chain(tmem + Cfg::T_A, sw128_desc(saddr(dys)), sw128_mn_desc(saddr(w3), 2048), 0, 0, 1, kk | B_MN, false);
+                mma_chain(tmem + Cfg::T_DW3, sw128_mn_desc(saddr(h2), 16384), sw128_mn_desc(saddr(dys), 16384), 128, 128,
+                          BM / 16, kk16 | A_MN | B_MN, !first);
+            }
+            mma_commit(&mma_bar);
+        }
+        products_done();
+        // dZ = dH o g'(Z) into h, its column sums into db
+        auto back = [&](uint32_t t0, const uint32_t (&gp)[16], unsigned char* h, float& db) {
+            float dz[32];
+#pragma unroll
+            for (int c = 0; c < 32; c += 16) {
+                float v[16];
+                __syncwarp();
+                tmem_ld16(taddr + t0 + (uint32_t)(cbeg + c), v);
+#pragma unroll
+                for (int k = 0; k < 16; k += 2) {
+                    const __nv_bfloat162 d2 = *reinterpret_cast<const __nv_bfloat162*>(&gp[(c + k) / 2]);
+                    v[k] *= __low2float(d2);
+                    v[k + 1] *= __high2float(d2);
+                    dz[c + k] = v[k];
+                    dz[c + k + 1] = v[k + 1];
+                }
+                store_h_sw128(h, r, cbeg + c, v);
+            }
+            db += column_sums32(dz, lane);
+        };
+        if (ok) back(Cfg::T_A, g2, h2, db2);
+        operands_ready();
+        if (tid == 0) {
+            if (ok) {
+                // dH1 = dZ2 W2 (contracts layer 2's units), dW2 += dZ2^T H1 (contracts the rows)
+#pragma unroll
+                for (int kc = 0; kc < 2; ++kc)
+                    mma_chain(tmem + Cfg::T_B, sw128_desc(saddr(h2) + kc * 16384),
+                              sw128_mn_desc(saddr(w2) + kc * 8192, 16384), 2, 128, BK / 16, kk | B_MN, kc > 0);
+                mma_chain(tmem + Cfg::T_DW2, sw128_mn_desc(saddr(h2), 16384), sw128_mn_desc(saddr(h1), 16384), 128, 128,
+                          BM / 16, kk | A_MN | B_MN, !first);
+            }
+            mma_commit(&mma_bar);
+        }
+        products_done();
+        if (ok) back(Cfg::T_B, g1, h1, db1);
+        operands_ready();
+        if (tid == 0) {
+            if (ok)  // dW1 += dZ1^T X
+                mma_chain(tmem + Cfg::T_DW1, sw128_mn_desc(saddr(h1), 16384), sw128_mn_desc(saddr(xs), 16384), 128, 128,
+                          BM / 16, idesc_bf16_f32(BM, NINP) | A_MN | B_MN, !first);
+            mma_commit(&mma_bar);
+        }
+        products_done();
+        if (tid == 0 && ok && tile + (int)gridDim.x < tiles) {
+            bar_expect_tx(&x_bar, Cfg::TX_X);
+            tma_load_2d(xs, &mx, &x_bar, 0, (tile + (int)gridDim.x) * BM);
+        }
+    }
+
+    if (ok) {
+        float* q = part + (size_t)blockIdx.x * Cfg::P_TOTAL;
+        float v[16];
+        auto drain = [&](uint32_t t0, float* row) {
+            __syncwarp();
+            tmem_ld16(taddr + t0, v);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                reinterpret_cast<float4*>(row)[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+        };
+        drain(Cfg::T_DW2 + cbeg, q + Cfg::P_W2 + r * NH + cbeg);
+        drain(Cfg::T_DW2 + cbeg + 16, q + Cfg::P_W2 + r * NH + cbeg + 16);
+        drain(Cfg::T_DW1 + cbeg / 2, q + Cfg::P_W1 + r * NINP + cbeg / 2);
+        if (warp < 4) {
+            __syncwarp();
+            tmem_ld16(taddr + Cfg::T_DW3, v);
+#pragma unroll
+            for (int k = 0; k < NOUTP; ++k) q[Cfg::P_W3 + k * NH + r] = v[k];
+            if (lane < NOUTP) q[Cfg::P_B3 + warp * NOUTP + lane] = db3;
+            if (lane == 0) loss_part[blockIdx.x * 4 + warp] = loss;
+        }
+        q[Cfg::P_B1 + (warp & 3) * NH + cbeg + lane] = db1;
+        q[Cfg::P_B2 + (warp & 3) * NH + cbeg + lane] = db2;
+    } else if (tid == 0) {
+        if (status) atomicOr(status, 1);
+        // let the loads started so far land before the CTA exits (bounded)
+        bar_wait(&w_bar, 0);
+        bar_wait(&x_bar, 0);
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) tmem_free(tmem, 512);
+}
+
 // ---- small kernels ---------------------------------------------------------------------------
 
-// x [rows][64] -> xt [64][rows]
-__global__ void transpose_x_kernel(const bf16* __restrict__ x, bf16* __restrict__ xt, int rows) {
-    __shared__ bf16 t[32][33];
-    const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
-    for (int k = threadIdx.y; k < 32; k += blockDim.y) t[k][threadIdx.x] = x[(size_t)(r0 + k) * NINP + c0 + threadIdx.x];
-    __syncthreads();
-    for (int k = threadIdx.y; k < 32; k += blockDim.y) xt[(size_t)(c0 + k) * rows + r0 + threadIdx.x] = t[threadIdx.x][k];
-}
-
-// grad[dst(r, c)] = sum over splits of part[s][r][c], r < 128, c < cols (fixed order).
-__global__ void reduce_partials_kernel(const float* __restrict__ part, int splits, int ld, int cols, float* __restrict__ grad,
-                                       int kind) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= BM * cols) return;
-    const int r = i / cols, c = i - r * cols;
-    float acc = 0.0f;
-    for (int s = 0; s < splits; ++s) acc += part[((size_t)s * BM + r) * ld + c];
-    if (kind == 0) {  // dW1: [128][64] -> W1[r][c], c < 54
-        if (c < NIN) grad[OFF_W1 + r * NIN + c] = acc;
-    } else if (kind == 1) {  // dW2
-        grad[OFF_W2 + r * NH + c] = acc;
-    } else {  // dW3^T: [128 h][16 o] -> W3[o][h], o < 12
-        if (c < NOUT) grad[OFF_W3 + c * NH + r] = acc;
+// grad[i] = the CTAs' partial sums in a fixed order: 64 parameters per block, four threads each
+// taking every fourth CTA; the last block sums the loss.
+__global__ void __launch_bounds__(256) reduce_gradient_kernel(const float* __restrict__ part,
+                                                              const double* __restrict__ loss_part, int ctas,
+                                                              float* __restrict__ grad, double* __restrict__ loss) {
+    using Cfg = TrainCfg;
+    __shared__ float sh[4][64];
+    pdl_launch_dependents();
+    pdl_wait();
+    const int t = threadIdx.x & 63, g = threadIdx.x >> 6;
+    if (blockIdx.x == gridDim.x - 1) {
+        if (threadIdx.x < 32) {
+            double l = 0.0;
+            for (int k = threadIdx.x; k < 4 * ctas; k += 32) l += __ldcg(loss_part + k);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) l += __shfl_down_sync(0xffffffffu, l, o);
+            if (threadIdx.x == 0) *loss = l;
+        }
+        return;
     }
+    const int i = blockIdx.x * 64 + t;
+    int off = 0, groups = 1, ld = 0;
+    if (i < OFF_B1) off = Cfg::P_W1 + (i / NIN) * NINP + i % NIN;
+    else if (i < OFF_W2) off = Cfg::P_B1 + i - OFF_B1, groups = 4, ld = NH;
+    else if (i < OFF_B2) off = Cfg::P_W2 + i - OFF_W2;
+    else if (i < OFF_W3) off = Cfg::P_B2 + i - OFF_B2, groups = 4, ld = NH;
+    else if (i < OFF_B3) off = Cfg::P_W3 + i - OFF_W3;
+    else off = Cfg::P_B3 + i - OFF_B3, groups = 4, ld = NOUTP;
+    float acc = 0.0f;
+    if (i < NPARAM) {
+#pragma unroll 8
+        for (int c = g; c < ctas; c += 4) acc += __ldcg(part + (size_t)c * Cfg::P_TOTAL + off);
+        for (int k = 1; k < groups; ++k)
+            for (int c = g; c < ctas; c += 4) acc += __ldcg(part + (size_t)c * Cfg::P_TOTAL + off + k * ld);
+    }
+    sh[g][t] = acc;
+    __syncthreads();
+    if (g == 0 && i < NPARAM) grad[i] = (sh[0][t] + sh[1][t]) + (sh[2][t] + sh[3][t]);
 }
 
-__global__ void adam_kernel(float* __restrict__ theta, float* __restrict__ m1, float* __restrict__ m2,
-                            const float* __restrict__ g, int n, float lr, float b1, float b2, float eps, float c1,
-                            float c2) {
+// The BF16 copy of parameter i in the layout the products read (zero padding where K or N is padded:
+// written once, when the network is created).
+__device__ __forceinline__ void cast_weight(int i, float v, bf16* w1p, bf16* w2, bf16* w3p) {
+    if (i < OFF_B1) w1p[(i / NIN) * NINP + i % NIN] = __float2bfloat16_rn(v);
+    else if (i >= OFF_W2 && i < OFF_B2) w2[i - OFF_W2] = __float2bfloat16_rn(v);
+    else if (i >= OFF_W3 && i < OFF_B3) w3p[i - OFF_W3] = __float2bfloat16_rn(v);
+}
+
+// One Adam step and the BF16 weights with it.
+__global__ void __launch_bounds__(256) adam_kernel(float* __restrict__ theta, float* __restrict__ m1, float* __restrict__ m2,
+                                                   const float* __restrict__ g, int n, float lr, float b1, float b2,
+                                                   float eps, float c1, float c2, bf16* __restrict__ w1p,
+                                                   bf16* __restrict__ w2, bf16* __restrict__ w3p) {
+    pdl_launch_dependents();
+    pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const float gi = g[i];
+    const float gi = __ldcg(g + i);
     const float a = b1 * m1[i] + (1.0f - b1) * gi;
     const float b = b2 * m2[i] + (1.0f - b2) * gi * gi;
     m1[i] = a;
     m2[i] = b;
-    theta[i] -= lr * (a / c1) / (sqrtf(b / c2) + eps);
+    const float t = theta[i] - lr * (a / c1) / (sqrtf(b / c2) + eps);
+    theta[i] = t;
+    cast_weight(i, t, w1p, w2, w3p);
 }
 
-// BF16 copies of the weights in the layouts the products read (zero padding where K or N is padded).
 __global__ void cast_weights_kernel(const float* __restrict__ th, bf16* __restrict__ w1p, bf16* __restrict__ w2,
-                                    bf16* __restrict__ w2t, bf16* __restrict__ w3p, bf16* __restrict__ w3tp) {
+                                    bf16* __restrict__ w3p) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < NH * NINP) {  // W1p [128][64]
-        const int r = i / NINP, c = i - r * NINP;
-        w1p[i] = __float2bfloat16_rn(c < NIN ? th[OFF_W1 + r * NIN + c] : 0.0f);
-    }
-    if (i < NH * NH) {  // W2 [128][128], W2^T
-        const int r = i / NH, c = i - r * NH;
-        const bf16 v = __float2bfloat16_rn(th[OFF_W2 + i]);
-        w2[i] = v;
-        w2t[c * NH + r] = v;
-    }
-    if (i < NOUTP * NH) {  // W3p [16][128]
-        const int o = i / NH, h = i - o * NH;
-        w3p[i] = __float2bfloat16_rn(o < NOUT ? th[OFF_W3 + o * NH + h] : 0.0f);
-    }
-    if (i < NH * NINP) {  // W3^T p [128][64]: [h][o]
-        const int h = i / NINP, o = i - h * NINP;
-        w3tp[i] = __float2bfloat16_rn(o < NOUT ? th[OFF_W3 + o * NH + h] : 0.0f);
-    }
+    if (i < NPARAM) cast_weight(i, th[i], w1p, w2, w3p);
 }
 
 }  // namespace
@@ -640,11 +729,11 @@ struct tvlbm_mlp {
     unsigned char* mem;
     size_t bytes;
     float *theta, *m1, *m2, *grad, *part;
-    double* loss;
+    double *loss, *loss_part;
     int* status;
-    bf16 *w1p, *w2, *w2t, *w3p, *w3tp;
-    bf16 *h1, *h1t, *g1, *h2, *h2t, *g2, *dy, *dyt, *dz2, *dz2t, *dz1t, *xt;
+    bf16 *w1p, *w2, *w3p;
     float* ybuf;
+    int ctas;  // most CTAs of a training pass (one per SM), the partial sums' extent
     int adam_t;
     unsigned long long uid;
     // descriptors of the last inference call (inputs at cached_x, cached_rows rows)
@@ -686,31 +775,6 @@ bool bf16_map(CUtensorMap* map, const void* base, int k_total, int rows, int ld,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int BN, int STAGES, class Epi>
-cudaError_t gemm(const CUtensorMap& ma, const CUtensorMap& mb, int row_tiles, int kchunks, int splits, int cps,
-                 const Epi& epi, int* status, cudaStream_t s) {
-    using Cfg = GemmCfg<BN, STAGES>;
-    static bool attr_set[64] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (!attr_set[dev]) {
-        const cudaError_t e = cudaFuncSetAttribute(gemm_kernel<BN, STAGES, Epi>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
-        if (e != cudaSuccess) return e;
-        attr_set[dev] = true;
-    }
-    gemm_kernel<BN, STAGES, Epi><<<dim3(row_tiles, splits), 128, Cfg::SMEM, s>>>(ma, mb, kchunks, cps, epi, status);
-    return cudaGetLastError();
-}
-
-// Split of kchunks K chunks over at most kMaxSplits CTAs (every split non-empty).
-void split_k(int kchunks, int* splits, int* cps) {
-    int s = kchunks < kMaxSplits ? kchunks : kMaxSplits;
-    *cps = (kchunks + s - 1) / s;
-    *splits = (kchunks + *cps - 1) / *cps;
-}
-
 int check_rows(tvlbm_mlp* m, int rows) {
     if (rows <= 0 || rows % BM || rows > m->max_rows)
         return mfail(m, TVLBM_EINVAL, "rows %d must be a positive multiple of 128 and at most %d", rows, m->max_rows);
@@ -730,7 +794,7 @@ int read_status(tvlbm_mlp* m) {
 }
 
 int refresh_weights(tvlbm_mlp* m) {
-    cast_weights_kernel<<<(NH * NH + 255) / 256, 256, 0, m->stream>>>(m->theta, m->w1p, m->w2, m->w2t, m->w3p, m->w3tp);
+    cast_weights_kernel<<<(NPARAM + 255) / 256, 256, 0, m->stream>>>(m->theta, m->w1p, m->w2, m->w3p);
     MLP_CUDA(m, cudaGetLastError(), "cast kernel");
     return TVLBM_OK;
 }
@@ -823,8 +887,10 @@ int tvlbm_mlp_create(int max_rows, tvlbm_mlp** out) {
     static std::atomic<unsigned long long> next_uid{1};
     m->uid = next_uid.fetch_add(1);
     const size_t R = (size_t)max_rows;
-    int splits = 0, cps = 0;
-    split_k(max_rows / BK, &splits, &cps);
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device);
+    if (sms < 1) sms = 1;
+    m->ctas = max_rows / BM < sms ? max_rows / BM : sms;
     // carve one allocation: FP32 block, then BF16 block (every piece 256-byte aligned)
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -833,14 +899,10 @@ int tvlbm_mlp_create(int max_rows, tvlbm_mlp** out) {
         return o;
     };
     const size_t o_theta = take(NPARAM * 4), o_m1 = take(NPARAM * 4), o_m2 = take(NPARAM * 4), o_grad = take(NPARAM * 4);
-    const size_t o_part = take((size_t)kMaxSplits * BM * NH * 4), o_loss = take(8), o_status = take(4);
+    const size_t o_part = take((size_t)m->ctas * TrainCfg::P_TOTAL * 4), o_losses = take((size_t)m->ctas * 4 * 8),
+                 o_loss = take(8), o_status = take(4);
     const size_t o_y = take(R * NOUTP * 4);
-    const size_t o_w1p = take(NH * NINP * 2), o_w2 = take(NH * NH * 2), o_w2t = take(NH * NH * 2),
-                 o_w3p = take(NOUTP * NH * 2), o_w3tp = take(NH * NINP * 2);
-    const size_t o_h1 = take(R * NH * 2), o_h1t = take(R * NH * 2), o_g1 = take(R * NH * 2), o_h2 = take(R * NH * 2),
-                 o_h2t = take(R * NH * 2), o_g2 = take(R * NH * 2), o_dy = take(R * NINP * 2),
-                 o_dyt = take(R * NOUTP * 2), o_dz2 = take(R * NH * 2), o_dz2t = take(R * NH * 2),
-                 o_dz1t = take(R * NH * 2), o_xt = take(R * NINP * 2);
+    const size_t o_w1p = take(NH * NINP * 2), o_w2 = take(NH * NH * 2), o_w3p = take(NOUTP * NH * 2);
     m->bytes = off;
     if (cudaMalloc((void**)&m->mem, off) != cudaSuccess) {
         delete m;
@@ -855,31 +917,16 @@ int tvlbm_mlp_create(int max_rows, tvlbm_mlp** out) {
     m->loss = (double*)(b + o_loss);
     m->status = (int*)(b + o_status);
     m->ybuf = (float*)(b + o_y);
+    m->loss_part = (double*)(b + o_losses);
     m->w1p = (bf16*)(b + o_w1p);
     m->w2 = (bf16*)(b + o_w2);
-    m->w2t = (bf16*)(b + o_w2t);
     m->w3p = (bf16*)(b + o_w3p);
-    m->w3tp = (bf16*)(b + o_w3tp);
-    m->h1 = (bf16*)(b + o_h1);
-    m->h1t = (bf16*)(b + o_h1t);
-    m->g1 = (bf16*)(b + o_g1);
-    m->h2 = (bf16*)(b + o_h2);
-    m->h2t = (bf16*)(b + o_h2t);
-    m->g2 = (bf16*)(b + o_g2);
-    m->dy = (bf16*)(b + o_dy);
-    m->dyt = (bf16*)(b + o_dyt);
-    m->dz2 = (bf16*)(b + o_dz2);
-    m->dz2t = (bf16*)(b + o_dz2t);
-    m->dz1t = (bf16*)(b + o_dz1t);
-    m->xt = (bf16*)(b + o_xt);
-    // zero everything once: parameters, moments, and the padded columns of dY (never written)
+    // zero everything once: parameters, moments, and the padding of the BF16 weights (never written)
     if (cudaMemset(m->mem, 0, off) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
         cudaFree(m->mem);
         delete m;
         return TVLBM_ECUDA;
     }
-    (void)splits;
-    (void)cps;
     *out = m;
     return TVLBM_OK;
 }
@@ -934,50 +981,25 @@ int tvlbm_mlp_loss_grad(tvlbm_mlp* m, const void* x, const float* ystar, int row
     if (rc) return rc;
     cudaSetDevice(m->device);
     cudaStream_t s = m->stream;
-    const int tiles = rows / BM;
-    CUtensorMap mx, mw1, mh1, mw2, mh2, mw3, mdy, mw3t, mdz2, mw2t, mdz1t, mxt, mdz2t, mh1t, mh2t, mdyt;
-    const bool okmaps =
-        bf16_map(&mx, x, NINP, rows, NINP, BM) && bf16_map(&mw1, m->w1p, NINP, NH, NINP, NH) &&
-        bf16_map(&mh1, m->h1, NH, rows, NH, BM) && bf16_map(&mw2, m->w2, NH, NH, NH, NH) &&
-        bf16_map(&mh2, m->h2, NH, rows, NH, BM) && bf16_map(&mw3, m->w3p, NH, NOUTP, NH, NOUTP) &&
-        bf16_map(&mdy, m->dy, NINP, rows, NINP, BM) && bf16_map(&mw3t, m->w3tp, NINP, NH, NINP, NH) &&
-        bf16_map(&mdz2, m->dz2, NH, rows, NH, BM) && bf16_map(&mw2t, m->w2t, NH, NH, NH, NH) &&
-        bf16_map(&mdz1t, m->dz1t, rows, NH, rows, BM) && bf16_map(&mxt, m->xt, rows, NINP, rows, NINP) &&
-        bf16_map(&mdz2t, m->dz2t, rows, NH, rows, BM) && bf16_map(&mh1t, m->h1t, rows, NH, rows, NH) &&
-        bf16_map(&mh2t, m->h2t, rows, NH, rows, BM) && bf16_map(&mdyt, m->dyt, rows, NOUTP, rows, NOUTP);
-    if (!okmaps) return mfail(m, TVLBM_EINVAL, "TMA descriptor rejected (alignment of x?)");
-    MLP_CUDA(m, cudaMemsetAsync(m->grad, 0, NPARAM * 4, s), "clear gradient");
-    MLP_CUDA(m, cudaMemsetAsync(m->loss, 0, 8, s), "clear loss");
-    transpose_x_kernel<<<dim3(rows / 32, NINP / 32), dim3(32, 8), 0, s>>>((const bf16*)x, m->xt, rows);
-    MLP_CUDA(m, cudaGetLastError(), "transpose");
-    // forward, keeping H, H^T and g'(Z)
-    EpiHidden e1{m->theta + OFF_B1, m->h1, m->h1t, m->g1, rows};
-    MLP_CUDA(m, (gemm<NH, 2>(mx, mw1, tiles, NINP / BK, 1, NINP / BK, e1, m->status, s)), "layer 1");
-    EpiHidden e2{m->theta + OFF_B2, m->h2, m->h2t, m->g2, rows};
-    MLP_CUDA(m, (gemm<NH, 2>(mh1, mw2, tiles, NH / BK, 1, NH / BK, e2, m->status, s)), "layer 2");
-    EpiOut e3{m->theta + OFF_B3, m->ybuf, ystar, m->dy, m->dyt, m->loss, m->grad + OFF_B3,
-              2.0f / ((float)rows * (float)NOUT), rows};
-    MLP_CUDA(m, (gemm<NOUTP, 2>(mh2, mw3, tiles, NH / BK, 1, NH / BK, e3, m->status, s)), "layer 3");
-    // back through the layers
-    EpiBack b2{m->g2, m->dz2, m->dz2t, m->grad + OFF_B2, rows};
-    MLP_CUDA(m, (gemm<NH, 2>(mdy, mw3t, tiles, NINP / BK, 1, NINP / BK, b2, m->status, s)), "dH2");
-    EpiBack b1{m->g1, nullptr, m->dz1t, m->grad + OFF_B1, rows};
-    MLP_CUDA(m, (gemm<NH, 2>(mdz2, mw2t, tiles, NH / BK, 1, NH / BK, b1, m->status, s)), "dH1");
-    // weight gradients: K = rows, split over CTAs, partials reduced in a fixed order
-    int splits = 0, cps = 0;
-    split_k(rows / BK, &splits, &cps);
-    EpiPartial p1{m->part, NINP};
-    MLP_CUDA(m, (gemm<NINP, 4>(mdz1t, mxt, 1, rows / BK, splits, cps, p1, m->status, s)), "dW1");
-    reduce_partials_kernel<<<(BM * NINP + 255) / 256, 256, 0, s>>>(m->part, splits, NINP, NINP, m->grad, 0);
-    MLP_CUDA(m, cudaGetLastError(), "reduce dW1");
-    EpiPartial p2{m->part, NH};
-    MLP_CUDA(m, (gemm<NH, 4>(mdz2t, mh1t, 1, rows / BK, splits, cps, p2, m->status, s)), "dW2");
-    reduce_partials_kernel<<<(BM * NH + 255) / 256, 256, 0, s>>>(m->part, splits, NH, NH, m->grad, 1);
-    MLP_CUDA(m, cudaGetLastError(), "reduce dW2");
-    EpiPartial p3{m->part, NOUTP};
-    MLP_CUDA(m, (gemm<NOUTP, 4>(mh2t, mdyt, 1, rows / BK, splits, cps, p3, m->status, s)), "dW3");
-    reduce_partials_kernel<<<(BM * NOUTP + 255) / 256, 256, 0, s>>>(m->part, splits, NOUTP, NOUTP, m->grad, 2);
-    MLP_CUDA(m, cudaGetLastError(), "reduce dW3");
+    const int tiles = rows / BM, ctas = tiles < m->ctas ? tiles : m->ctas;
+    CUtensorMap mx, mw1, mw2, mw3;
+    if (!bf16_map(&mx, x, NINP, rows, NINP, BM) || !bf16_map(&mw1, m->w1p, NINP, NH, NINP, NH) ||
+        !bf16_map(&mw2, m->w2, NH, NH, NH, NH) || !bf16_map(&mw3, m->w3p, NH, NOUTP, NH, NOUTP))
+        return mfail(m, TVLBM_EINVAL, "TMA descriptor rejected (alignment of x?)");
+    if ((uintptr_t)ystar & 15) return mfail(m, TVLBM_EINVAL, "ystar must be 16-byte aligned");
+    static bool attr_set[64] = {};
+    if (m->device < 0 || m->device >= 64 || !attr_set[m->device]) {
+        MLP_CUDA(m, cudaFuncSetAttribute(mlp_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TrainCfg::SMEM),
+                 "training kernel attribute");
+        if (m->device >= 0 && m->device < 64) attr_set[m->device] = true;
+    }
+    MLP_CUDA(m, launch_pdl(mlp_train_kernel, dim3(ctas), dim3(kFusedThreads), TrainCfg::SMEM, s, mx, mw1, mw2, mw3,
+                           (const float*)m->theta, ystar, tiles, 2.0f / ((float)rows * (float)NOUT), m->part, m->loss_part,
+                           m->status),
+             "training pass");
+    MLP_CUDA(m, launch_pdl(reduce_gradient_kernel, dim3((NPARAM + 63) / 64 + 1), dim3(256), 0, s, (const float*)m->part,
+                           (const double*)m->loss_part, ctas, m->grad, m->loss),
+             "gradient reduction");
     if (loss || grad) {
         double l = 0.0;
         if (loss) MLP_CUDA(m, cudaMemcpyAsync(&l, m->loss, 8, cudaMemcpyDeviceToHost, s), "copy loss");
@@ -995,10 +1017,10 @@ int tvlbm_mlp_adam(tvlbm_mlp* m, float lr, float beta1, float beta2, float eps) 
     cudaSetDevice(m->device);
     m->adam_t += 1;
     const float c1 = 1.0f - powf(beta1, (float)m->adam_t), c2 = 1.0f - powf(beta2, (float)m->adam_t);
-    adam_kernel<<<(NPARAM + 255) / 256, 256, 0, m->stream>>>(m->theta, m->m1, m->m2, m->grad, NPARAM, lr, beta1, beta2,
-                                                             eps, c1, c2);
-    MLP_CUDA(m, cudaGetLastError(), "adam kernel");
-    return refresh_weights(m);
+    MLP_CUDA(m, launch_pdl(adam_kernel, dim3((NPARAM + 255) / 256), dim3(256), 0, m->stream, m->theta, m->m1, m->m2,
+                           (const float*)m->grad, NPARAM, lr, beta1, beta2, eps, c1, c2, m->w1p, m->w2, m->w3p),
+             "adam kernel");
+    return TVLBM_OK;
 }
 
 const char* tvlbm_mlp_last_error(const tvlbm_mlp* m) { return m ? m->err : "null network"; }

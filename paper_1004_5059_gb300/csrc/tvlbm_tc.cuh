@@ -106,8 +106,22 @@ __device__ __forceinline__ uint64_t sw128_desc(uint32_t smem_byte_addr) {
     return d;
 }
 
+// The same layout read as an MN-major operand (the contraction runs over the tile's rows): 64
+// consecutive entries of M or N per 128-byte row, the next 64 `chunk_bytes` further (leading byte
+// offset), 8 rows of K per 1024 bytes (stride byte offset).  The k-th 16-row slice starts 2048 k bytes
+// further.
+__device__ __forceinline__ uint64_t sw128_mn_desc(uint32_t smem_byte_addr, uint32_t chunk_bytes) {
+    uint64_t d = 0;
+    d |= (uint64_t)((smem_byte_addr >> 4) & 0x3FFFu);
+    d |= (uint64_t)((chunk_bytes >> 4) & 0x3FFFu) << 16;
+    d |= (uint64_t)((1024u >> 4) & 0x3FFFu) << 32;
+    d |= (uint64_t)1u << 46;
+    d |= (uint64_t)2u << 61;
+    return d;
+}
+
 // Instruction descriptor of kind::f16: FP32 accumulator (bits 4-5 = 1), A and B BF16 (bits 7-9
-// and 10-12 = 1), both K-major (bits 15, 16 = 0), N >> 3 in bits 17-22, M >> 4 in bits 24-28.
+// and 10-12 = 1), both K-major (bits 15, 16 = 0; set for an MN-major A, B), N >> 3 in bits 17-22, M >> 4 in bits 24-28.
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
