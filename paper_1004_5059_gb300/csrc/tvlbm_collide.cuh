@@ -235,6 +235,136 @@ __device__ __forceinline__ void cell_collide_dev(float (&s)[N1 * N1], const KPar
     }
 }
 
+// ---- FP64 full populations ---------------------------------------------------------------------
+// An FP64 warp instruction takes 64 cycles of its SM partition, so the collision counts them: moments
+// from mirror pairs (x_m = -x_i, w_m = w_i), the even and odd parts of the equilibrium shared by a
+// pair, one multiply-add each for the equilibrium's excess and the relaxation (about 240 instructions
+// per cell of D2Q16, gather included, where the untransformed sums took 400).  In pieces per y-node,
+// so that the lanes of a cell shared by several lanes run the same operations; the rounding is
+// spelled out (no contraction), so that every form gets the same bits.
+// Row sums of y-node j: r = sum s, rx = sum x_i s, q = sum (x_i^2 + x_j^2) s.
+template <int N1>
+__device__ __forceinline__ void f64_row_sums(const double (&v)[N1], const KParams& p, double x2j, double& r, double& rx,
+                                             double& q) {
+    constexpr int H = N1 / 2;
+    double rxx = 0.0;
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+        const int m = N1 - 1 - i;
+        const double a = __dadd_rn(v[i], v[m]), b = __dadd_rn(v[m], -v[i]);
+        r = i == 0 ? a : __dadd_rn(r, a);
+        rx = i == 0 ? __dmul_rn(p.xd[m], b) : fma(p.xd[m], b, rx);
+        rxx = i == 0 ? __dmul_rn(p.x2d[m], a) : fma(p.x2d[m], a, rxx);
+    }
+    if (N1 & 1) r = __dadd_rn(r, v[H]);
+    q = fma(x2j, r, rxx);
+}
+// The cell's factors from the rows' sums: density, Hermite factors, and per x-pair the even and odd
+// sums of the x part (1 + X_i2 + .., X_i1 + X_i3 + ..) and X_ia, a < N.
+template <int N1>
+struct F64Cell {
+    static constexpr int N = N1 - 1, H = N1 / 2, HC = (N1 + 1) / 2;
+    double rho, hy[N + 1], X[HC][N], ev[HC], od[HC];
+    __device__ __forceinline__ void set(const double (&r)[N1], const double (&rx)[N1], const double (&q)[N1], const KParams& p) {
+        double m0 = 0.0, mx = 0.0, my = 0.0, me = 0.0;
+#pragma unroll
+        for (int j = 0; j < H; ++j) {
+            const int m = N1 - 1 - j;
+            const double a = __dadd_rn(r[j], r[m]), b = __dadd_rn(r[m], -r[j]);
+            const double c = __dadd_rn(rx[j], rx[m]), d = __dadd_rn(q[j], q[m]);
+            m0 = j == 0 ? a : __dadd_rn(m0, a);
+            mx = j == 0 ? c : __dadd_rn(mx, c);
+            me = j == 0 ? d : __dadd_rn(me, d);
+            my = j == 0 ? __dmul_rn(p.xd[m], b) : fma(p.xd[m], b, my);
+        }
+        if (N1 & 1) {
+            m0 = __dadd_rn(m0, r[H]);
+            mx = __dadd_rn(mx, rx[H]);
+            me = __dadd_rn(me, q[H]);
+        }
+        rho = m0;
+        const double inv = 1.0 / rho, ux = __dmul_rn(mx, inv), uy = __dmul_rn(my, inv);
+        const double th = fma(0.5, fma(me, inv, -fma(ux, ux, __dmul_rn(uy, uy))), -1.0);
+        double hx[N + 1];
+        hx[0] = hy[0] = 1.0;
+        hx[1] = ux;
+        hy[1] = uy;
+#pragma unroll
+        for (int n = 1; n < N; ++n) {
+            const double nth = n == 1 ? th : __dmul_rn((double)n, th);
+            hx[n + 1] = n == 1 ? fma(ux, ux, th) : fma(ux, hx[n], __dmul_rn(nth, hx[n - 1]));
+            hy[n + 1] = n == 1 ? fma(uy, uy, th) : fma(uy, hy[n], __dmul_rn(nth, hy[n - 1]));
+        }
+#pragma unroll
+        for (int i = 0; i < HC; ++i) {
+            ev[i] = 1.0;
+            od[i] = 0.0;
+#pragma unroll
+            for (int a = 1; a <= N; ++a) {
+                if ((N1 & 1) && i == H && (a & 1)) {  // the node 0 has no odd part
+                    if (a < N) X[i][a] = 0.0;
+                    continue;
+                }
+                if (a < N) {
+                    X[i][a] = __dmul_rn(hx[a], p.Ed[i][a]);
+                    if (a & 1) od[i] = a == 1 ? X[i][a] : __dadd_rn(od[i], X[i][a]);
+                    else ev[i] = __dadd_rn(ev[i], X[i][a]);
+                } else {
+                    if (a & 1) od[i] = fma(hx[a], p.Ed[i][a], od[i]);
+                    else ev[i] = fma(hx[a], p.Ed[i][a], ev[i]);
+                }
+            }
+        }
+    }
+    // Relax the populations of y-node j: v += om (w rho (1 + phi) - v).
+    __device__ __forceinline__ void relax(double (&v)[N1], int j, const KParams& p, double om) const {
+        double P[N + 1];
+        P[1] = __dmul_rn(hy[1], p.Ed[j][1]);
+#pragma unroll
+        for (int a = 2; a <= N; ++a) P[a] = fma(hy[a], p.Ed[j][a], P[a - 1]);
+#pragma unroll
+        for (int i = 0; i < HC; ++i) {
+            const int m = N1 - 1 - i;
+            double e = __dadd_rn(ev[i], P[N]), o = od[i];
+#pragma unroll
+            for (int a = 1; a < N; ++a) {
+                if (a & 1) {
+                    if (i != m) o = fma(X[i][a], P[N - a], o);
+                } else {
+                    e = fma(X[i][a], P[N - a], e);
+                }
+            }
+            const double W = __dmul_rn(p.wwd[i + N1 * j], rho);
+            if (i == m) {
+                v[i] = fma(om, fma(W, e, -v[i]), v[i]);
+            } else {
+                v[i] = fma(om, fma(W, __dadd_rn(e, o), -v[i]), v[i]);
+                v[m] = fma(om, fma(W, __dadd_rn(e, -o), -v[m]), v[m]);
+            }
+        }
+    }
+};
+template <int N1>
+__device__ __forceinline__ void cell_collide_f64(double (&s)[N1 * N1], const KParams& p, double om) {
+    double r[N1], rx[N1], q[N1], v[N1];
+#pragma unroll
+    for (int j = 0; j < N1; ++j) {
+#pragma unroll
+        for (int i = 0; i < N1; ++i) v[i] = s[i + N1 * j];
+        f64_row_sums<N1>(v, p, p.x2d[j], r[j], rx[j], q[j]);
+    }
+    F64Cell<N1> c;
+    c.set(r, rx, q, p);
+#pragma unroll
+    for (int j = 0; j < N1; ++j) {
+#pragma unroll
+        for (int i = 0; i < N1; ++i) v[i] = s[i + N1 * j];
+        c.relax(v, j, p, om);
+#pragma unroll
+        for (int i = 0; i < N1; ++i) s[i + N1 * j] = v[i];
+    }
+}
+
 // Collision for full FP32 populations.  s holds the gathered s_l = f_l - Whi_l, the population
 // less the float Whi_l of its rest value w_l (exact while f_l stays within a factor 2 of it), and
 // leaves holding f*_l.  The collision takes the state for f'_l = f_l + (w_l - Whi_l): a constant
@@ -295,14 +425,20 @@ __device__ __forceinline__ void cell_collide_split(float (&s)[N1 * N1], const KP
     const float ux = mx * inv, uy = my * inv;
     const float th = 0.5f * ((me - 2.0f * m0) * inv - (ux * ux + uy * uy));
 
-    float hx[N + 1], hy[N + 1];
-    hx[0] = hy[0] = 1.f;
-    hx[1] = ux;
-    hy[1] = uy;
+    // Hermite factors of both axes in packed pairs (x, y), as in cell_collide_dev
+    float2 hxy[N + 1];
+    hxy[0] = make_float2(1.f, 1.f);
+    hxy[1] = make_float2(ux, uy);
 #pragma unroll
     for (int n = 1; n < N; ++n) {
-        hx[n + 1] = fmaf(ux, hx[n], (float)n * th * hx[n - 1]);
-        hy[n + 1] = fmaf(uy, hy[n], (float)n * th * hy[n - 1]);
+        const float nth = (float)n * th;
+        hxy[n + 1] = __ffma2_rn(hxy[1], hxy[n], __fmul2_rn(make_float2(nth, nth), hxy[n - 1]));
+    }
+    float hx[N + 1], hy[N + 1];
+#pragma unroll
+    for (int n = 0; n <= N; ++n) {
+        hx[n] = hxy[n].x;
+        hy[n] = hxy[n].y;
     }
 
     // first-order cancellation of the float node tables' defects
@@ -334,29 +470,58 @@ __device__ __forceinline__ void cell_collide_split(float (&s)[N1 * N1], const KP
 #pragma unroll
     for (int i = 0; i < (ODD ? H + 1 : H); ++i) {
         const int m = N1 - 1 - i;
-        float se = 0.f, so = 0.f, pe = 0.f, po = 0.f;
+        float2 exy = make_float2(0.f, 0.f), oxy = make_float2(0.f, 0.f);
 #pragma unroll
         for (int a = 1; a <= N; ++a) {
-            const float xa = hx[a] * p.Ef[i][a];
-            const float ya = hy[a] * p.Ef[i][a];
-            if (a & 1) { so += xa; po += ya; } else { se += xa; pe += ya; }
-            P[i][a] = pe + po;
-            P[m][a] = pe - po;
+            const float2 e2 = make_float2(p.Ef[i][a], p.Ef[i][a]);
+            if (a & 1) oxy = __ffma2_rn(hxy[a], e2, oxy); else exy = __ffma2_rn(hxy[a], e2, exy);
+            P[i][a] = exy.y + oxy.y;
+            P[m][a] = exy.y - oxy.y;
             if (a < N) {
-                Xp[i][a] = orho * xa;
+                Xp[i][a] = orho * (hx[a] * p.Ef[i][a]);
                 Xp[m][a] = (a & 1) ? -Xp[i][a] : Xp[i][a];
             }
         }
         const float cx2 = 0.5f * G * p.x2f[i];
         const float ci = fmaf(Dx, p.xf[i], cx2), cim = fmaf(-Dx, p.xf[i], cx2);
         const float cj = fmaf(Dy, p.xf[i], cx2), cjm = fmaf(-Dy, p.xf[i], cx2);
-        A[i] = fmaf(orho, se + so, -om * ci);
-        A[m] = fmaf(orho, se - so, -om * cim);
+        A[i] = fmaf(orho, exy.x + oxy.x, -om * ci);
+        A[m] = fmaf(orho, exy.x - oxy.x, -om * cim);
         B[i] = fmaf(orho, P[i][N], -om * cj);
         B[m] = fmaf(orho, P[m][N], -om * cjm);
     }
     const float wdr = om * (m0 - (Dm - G));
     const float keep = 1.f - om;
+    if constexpr (!ODD) {
+        // mirror pairs (i, n-1-i), whose weights are equal, in packed FP32 pairs
+        float2 A2[H], X2[H][N > 1 ? N : 1];
+#pragma unroll
+        for (int i = 0; i < H; ++i) {
+            A2[i] = make_float2(A[i], A[N1 - 1 - i]);
+#pragma unroll
+            for (int a = 1; a < N; ++a) X2[i][a] = make_float2(Xp[i][a], Xp[N1 - 1 - i][a]);
+        }
+        const float2 keep2 = make_float2(keep, keep);
+#pragma unroll
+        for (int j = 0; j < N1; ++j) {
+            const float bj = B[j] + wdr;
+            const float2 bj2 = make_float2(bj, bj);
+#pragma unroll
+            for (int i = 0; i < H; ++i) {
+                const int l = i + N1 * j, lm = N1 - 1 - i + N1 * j;
+                float2 w2 = __fadd2_rn(A2[i], bj2);
+#pragma unroll
+                for (int a = 1; a < N; ++a) w2 = __ffma2_rn(X2[i][a], make_float2(P[j][N - a], P[j][N - a]), w2);
+                const float2 hi = make_float2(p.Whi[l], p.Whi[lm]);
+                const float2 t = __ffma2_rn(keep2, make_float2(s[l], s[lm]),
+                                            __ffma2_rn(hi, w2, __fmul2_rn(make_float2(p.Wlo[l], p.Wlo[lm]), w2)));
+                const float2 o = __fadd2_rn(hi, t);
+                s[l] = o.x;
+                s[lm] = o.y;
+            }
+        }
+        return;
+    }
 #pragma unroll
     for (int j = 0; j < N1; ++j) {
         const float bj = B[j] + wdr;

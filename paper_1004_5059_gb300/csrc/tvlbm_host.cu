@@ -255,6 +255,8 @@ void fill_kparams(KParams& p, const Rule& r, int N, double dt, double tau, doubl
             p.Ef[i][k] = (float)p.Ed[i][k];
         }
     }
+    for (int j = 0; j < r.n; ++j)
+        for (int i = 0; i < r.n; ++i) p.wwd[i + r.n * j] = r.w[i] * r.w[j];
     // Mirror nodes +-x share one overlap fraction pair alpha(-x) = 1 - alpha(x); keep that exact
     // in float (the member >= 1/2 is rounded, the other is 1 minus it, exact by Sterbenz).
     for (int i = 0; i < r.n; ++i) {

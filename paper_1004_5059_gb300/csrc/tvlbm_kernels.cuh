@@ -65,6 +65,7 @@ struct KParams {
     float xf[kMaxN1], wf[kMaxN1], af[kMaxN1];
     double xd[kMaxN1], wd[kMaxN1], ad[kMaxN1];
     double x2d[kMaxN1];  // xd * xd
+    double wwd[kMaxQ];   // wd_i * wd_j of velocity l = i + n j
     float Ef[kMaxN1][kMaxN1];
     double Ed[kMaxN1][kMaxN1];
     float x2f[kMaxN1];   // float(xf * xf)

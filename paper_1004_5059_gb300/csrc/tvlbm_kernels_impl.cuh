@@ -6,6 +6,7 @@
 #include "tvlbm_strip.cuh"
 #include "tvlbm_tiled.cuh"
 
+
 namespace tvlbm {
 
 // =============================================================================================
@@ -49,6 +50,91 @@ __global__ void __launch_bounds__(256) sweep_plain_kernel(const typename C::T* _
     const Geom g = geom_of(p);
     collide_cell<N1, C, ROWS>(s, p, g, y);
     store_collided<N1, C>(fout, g, x, y, s);
+}
+
+// FP64 on a small grid: a cell shared by LG lanes (4 for D2Q9 and D2Q16, 8 for D2Q36), lane j taking the
+// populations of y-node j.  An FP64 warp instruction takes 64 cycles of its SM partition whatever its
+// active lanes, and the chip has 608 partitions; one cell per lane would leave most of them idle
+// (64 x 64 cells: 128 warps of 245 instructions, 14.6 us per step; here 512 of about 105).  The row
+// sums meet by shuffles, the shared factors are computed by every lane.  The arithmetic is
+// collide_cell's, piece by piece: the same bits as the other forms.
+template <int N1>
+__global__ void __launch_bounds__(32) sweep_lanes_kernel(const double* __restrict__ fin, double* __restrict__ fout,
+                                                         const KParams p) {
+    constexpr int LG = N1 <= 4 ? 4 : 8, CELLS = 32 / LG;
+    pdl_launch_dependents();
+    pdl_wait();
+    const int gx = (p.nx + CELLS - 1) / CELLS, y = blockIdx.x / gx, lane = threadIdx.x;
+    const int x = (blockIdx.x - y * gx) * CELLS + lane / LG, xl = min(x, p.nx - 1);
+    const int j = min(lane % LG, N1 - 1), first = lane - lane % LG;
+    const double ay = p.ad[j];
+    const double* b = fin + (long long)(N1 * j) * p.plane + (long long)(y + HY - p.sh[j]) * p.pitch + (xl + p.hx);
+    double v[N1];
+#pragma unroll
+    for (int i = 0; i < N1; ++i) {
+        const double* c = b + (long long)i * p.plane - p.sh[i];
+        const double v00 = __ldg(c), v01 = __ldg(c - 1), v10 = __ldg(c - p.pitch), v11 = __ldg(c - p.pitch - 1);
+        const double r0 = fma(p.ad[i], __dadd_rn(v01, -v00), v00), r1 = fma(p.ad[i], __dadd_rn(v11, -v10), v10);
+        v[i] = fma(ay, __dadd_rn(r1, -r0), r0);
+    }
+    double r, rx, q, ra[N1], rxa[N1], qa[N1];
+    f64_row_sums<N1>(v, p, p.x2d[j], r, rx, q);
+#pragma unroll
+    for (int k = 0; k < N1; ++k) {
+        ra[k] = __shfl_sync(0xffffffffu, r, first + k);
+        rxa[k] = __shfl_sync(0xffffffffu, rx, first + k);
+        qa[k] = __shfl_sync(0xffffffffu, q, first + k);
+    }
+    F64Cell<N1> cell;
+    cell.set(ra, rxa, qa, p);
+    cell.relax(v, j, p, p.omegad);
+    if (x >= p.nx || lane % LG >= N1) return;
+    // the cell's position and its periodic images in the read frame (see store_collided)
+    const Geom g = geom_of(p);
+    const int x0 = x - g.nx * ((x + FILL) / g.nx), y0 = g.walls ? y : y - g.ny * ((y + FILL) / g.ny);
+    const int y1 = g.walls ? y + 1 : g.ny + FILL;
+    for (int yy = y0; yy < y1; yy += g.ny)
+        for (int xx = x0; xx < g.nx + FILL; xx += g.nx) {
+            double* o = fout + (long long)(N1 * j) * g.plane + (long long)(yy + HY) * g.pitch + (xx + g.hx);
+#pragma unroll
+            for (int i = 0; i < N1; ++i) {
+                stg(o, v[i]);
+                o += g.plane;
+            }
+        }
+}
+
+// The tiled form runs small domains without tiles (the same bits).  A tile's windows take a TMA round
+// trip and its threads walk 2 to 4 rows one after another, which a small grid has no other work to
+// hide: 100 x 75 D2Q9 FP32 4.9 us per step tiled against 2.5 with one cell per thread, 128 x 128
+// D2Q16 6.4 against 2.9.  The line lies where the tiles' fewer loads (each value once, not four times
+// through the L1 cache) begin to pay: at 12 M populations in 4-byte storage (768 x 768 D2Q16 15.3
+// against 16.8 us, 1000 x 601 17.5 against 19.0; 1024 x 1024 30.8 against 30.7) and 8 M in 2-byte
+// storage, whose single loads carry half as much (600 x 600 D2Q16 11.0 against 11.6 us; 1024 x 512
+// D2Q36 40 against 35.5).  FP64 is bound by its arithmetic, so what counts is an even spread over the
+// SM partitions: blocks of one warp, launched without programmatic overlap (blocks placed around those
+// of a kernel still resident share partitions: 64 x 64 D2Q16 8.5 instead of 5.6 us, 256 x 256 59
+// instead of 37), up to 600 cells per SM (256 x 256 37 against 51 to 72 us tiled; 500 x 300 79.7 against
+// 76.3), and lanes sharing a cell up to 64 cells per SM (32 for D2Q36, whose cells take 8 lanes): 64 x
+// 64 D2Q16 5.6 against 11.8 us with one lane per cell, 128 x 80 10.7 with one.
+inline int sm_count() {
+    static int sms[64] = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64) return 0;
+    if (!sms[dev]) cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev);
+    return sms[dev];
+}
+template <int N1, class C>
+inline bool sweep_without_tiles(const KParams& p) {
+    const long long cells = (long long)p.nx * p.ny;
+    if (p.ny > 65535) return false;  // rows of blocks: the grid's y extent
+    if (sizeof(typename C::T) == 8) return cells <= 600LL * sm_count();
+    return cells * (N1 * N1) <= (sizeof(typename C::T) == 4 ? 12000000LL : 8000000LL);
+}
+template <int N1>
+inline bool sweep_in_lanes(const KParams& p) {
+    return (long long)p.nx * p.ny <= (N1 <= 4 ? 64LL : 32LL) * sm_count();
 }
 
 // =============================================================================================
@@ -488,13 +574,23 @@ struct Launch {
     static cudaError_t sweep_c(int form, int cfg, const void* fin, void* fout, const SweepMaps* maps, const KParams& p,
                                cudaStream_t s) {
         using T = typename C::T;
-        if (form == FORM_TILED) return tiled_sweep<N1, C>(cfg, maps, (T*)fout, p, s);
+        const bool small = form == FORM_TILED && sweep_without_tiles<N1, C>(p);
+        if (form == FORM_TILED && !small) return tiled_sweep<N1, C>(cfg, maps, (T*)fout, p, s);
         if (form == FORM_STRIP) return strip_sweep<N1, C>(maps, (T*)fout, p, s);
-        const dim3 b(32, 8);
+        constexpr bool F64 = sizeof(T) == 8;
+        if constexpr (F64) {
+            constexpr int CELLS = N1 <= 4 ? 8 : 4;
+            if (small && sweep_in_lanes<N1>(p))
+                return launch_as(false, sweep_lanes_kernel<N1>, dim3((unsigned)((p.nx + CELLS - 1) / CELLS * p.ny)),
+                                 dim3(32), 0, s, (const T*)fin, (T*)fout, p);
+        }
+        // blocks of 128 threads: 3 to 8 % faster than 256 from 128 x 128 to 1024 x 1024 (D2Q36 channels
+        // up to 30 %); one warp in FP64 (see above)
+        const dim3 b(32, p.ny > 4 * 65535 ? 8 : (F64 && p.ny <= 65535) ? 1 : 4);
         if constexpr (C::dev) {
             if (p.rowf) return launch_pdl(sweep_plain_kernel<N1, C, true>, grid2d(p, b), b, 0, s, (const T*)fin, (T*)fout, p);
         }
-        return launch_pdl(sweep_plain_kernel<N1, C, false>, grid2d(p, b), b, 0, s, (const T*)fin, (T*)fout, p);
+        return launch_as(!F64, sweep_plain_kernel<N1, C, false>, grid2d(p, b), b, 0, s, (const T*)fin, (T*)fout, p);
     }
     template <class C>
     static cudaError_t init_c(const double* fields, void* f, const KParams& p, cudaStream_t s) {

@@ -238,8 +238,7 @@ __device__ __forceinline__ void collide_cell(typename C::R (&s)[N1 * N1], const 
         }
     }
     else if constexpr (C::split) cell_collide_split<N1>(s, p, g.omegaf);
-    else if constexpr (std::is_same<typename C::R, double>::value) cell_collide<N1, false, double>(s, p, g.omegad);
-    else cell_collide<N1, false, float>(s, p, g.omegaf);
+    else cell_collide_f64<N1>(s, p, g.omegad);
 }
 
 // Store one collided cell.  A cell within FILL of a periodic edge is stored at every position it
