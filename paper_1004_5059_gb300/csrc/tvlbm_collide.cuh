@@ -492,8 +492,9 @@ __device__ __forceinline__ void cell_collide_split(float (&s)[N1 * N1], const KP
     }
     const float wdr = om * (m0 - (Dm - G));
     const float keep = 1.f - om;
-    if constexpr (!ODD) {
-        // mirror pairs (i, n-1-i), whose weights are equal, in packed FP32 pairs
+    if constexpr (!ODD && N1 <= 4) {
+        // mirror pairs (i, n-1-i), whose weights are equal, in packed FP32 pairs (D2Q36: the pairs' copies
+        // spill in the dataflow kernel)
         float2 A2[H], X2[H][N > 1 ? N : 1];
 #pragma unroll
         for (int i = 0; i < H; ++i) {
