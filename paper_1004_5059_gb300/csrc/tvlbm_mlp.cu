@@ -44,58 +44,62 @@ using bf16 = __nv_bfloat16;
 // GELU g(z) = z Phi(z), Phi(z) = (1 + erf(z / sqrt 2)) / 2, and g'(z) = Phi(z) + z phi(z).  erf by
 // the rational approximation of Abramowitz & Stegun, Handbook of Mathematical Functions, eq.
 // 7.1.26 (after Hastings): erf(x) = 1 - (a1 t + ... + a5 t^5) exp(-x^2), t = 1 / (1 + p x), x >= 0,
-// |error| <= 1.5e-7, odd in x; the reciprocal and the exponential by the hardware approximations.
-// The network stores its activations in BF16 (relative step 2^-8), so the error is invisible.
-// E2 = exp(-x^2) = exp(-z^2 / 2) also gives phi(z) = E2 / sqrt(2 pi).
+// |error| <= 1.5e-7, odd in x; the reciprocal and the exponential (2^(s log2 e)) by the hardware's
+// approximations without the handling of subnormal results (1 + p x >= 1; an exp(-x^2) that small adds
+// nothing to 1).  The network stores its activations in BF16 (relative step 2^-8), so the error is
+// invisible.  E2 = exp(-x^2) = exp(-z^2 / 2) also gives phi(z) = E2 / sqrt(2 pi).
+__device__ __forceinline__ float rcp_approx(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float ex2_approx(float x) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+constexpr float kLog2e = 1.4426950408889634f;
 __device__ __forceinline__ float erf_as(float x, float& e2) {
     const float ax = fabsf(x);
-    const float t = __fdividef(1.0f, fmaf(0.3275911f, ax, 1.0f));
+    const float t = rcp_approx(fmaf(0.3275911f, ax, 1.0f));
     const float poly =
         t * fmaf(t, fmaf(t, fmaf(t, fmaf(t, 1.061405429f, -1.453152027f), 1.421413741f), -0.284496736f), 0.254829592f);
-    e2 = __expf(-ax * ax);
+    e2 = ex2_approx(__fmul_rn(__fmul_rn(ax, ax), -kLog2e));
     return copysignf(fmaf(-poly, e2, 1.0f), x);
 }
 __device__ __forceinline__ float gelu_f(float z) {
     float e2;
     return 0.5f * z * (1.0f + erf_as(z * 0.70710678118654752f, e2));
 }
-// Two GELUs in packed FP32 pairs, per lane the operations of gelu_f in its order (a packed
-// multiply, add or fused multiply-add rounds each lane as the scalar instruction; the
-// reciprocal, the exponential, |x| and the sign stay scalar).  The forward epilogues and
-// tvlbm_mlp_activation's g use it.
-__device__ __forceinline__ float2 gelu2_f(float2 z) {
-    const float2 x = __fmul2_rn(z, make_float2(0.70710678118654752f, 0.70710678118654752f));
+// The same for a pair in packed FP32, per lane the operations of erf_as in their order (a packed
+// multiply, add or fused multiply-add rounds each lane as the scalar instruction; the reciprocal,
+// the exponential, |x| and the sign stay scalar; the polynomial's sign is in its coefficients):
+// 1 + erf(x), and exp(-x^2).
+__device__ __forceinline__ float2 erf2_plus1(float2 x, float2& e2) {
     const float2 ax = make_float2(fabsf(x.x), fabsf(x.y));
     const float2 d = __ffma2_rn(make_float2(0.3275911f, 0.3275911f), ax, make_float2(1.0f, 1.0f));
-    const float2 t = make_float2(__fdividef(1.0f, d.x), __fdividef(1.0f, d.y));
-    float2 q = __ffma2_rn(t, make_float2(1.061405429f, 1.061405429f), make_float2(-1.453152027f, -1.453152027f));
-    q = __ffma2_rn(t, q, make_float2(1.421413741f, 1.421413741f));
-    q = __ffma2_rn(t, q, make_float2(-0.284496736f, -0.284496736f));
-    q = __ffma2_rn(t, q, make_float2(0.254829592f, 0.254829592f));
-    const float2 poly = __fmul2_rn(t, q);
-    const float2 sq = __fmul2_rn(make_float2(-ax.x, -ax.y), ax);
-    const float2 e2 = make_float2(__expf(sq.x), __expf(sq.y));
-    const float2 r = __ffma2_rn(make_float2(-poly.x, -poly.y), e2, make_float2(1.0f, 1.0f));
-    const float2 er = make_float2(copysignf(r.x, x.x), copysignf(r.y, x.y));
-    return __fmul2_rn(__fmul2_rn(make_float2(0.5f, 0.5f), z), __fadd2_rn(make_float2(1.0f, 1.0f), er));
+    const float2 t = make_float2(rcp_approx(d.x), rcp_approx(d.y));
+    float2 q = __ffma2_rn(t, make_float2(-1.061405429f, -1.061405429f), make_float2(1.453152027f, 1.453152027f));
+    q = __ffma2_rn(t, q, make_float2(-1.421413741f, -1.421413741f));
+    q = __ffma2_rn(t, q, make_float2(0.284496736f, 0.284496736f));
+    q = __ffma2_rn(t, q, make_float2(-0.254829592f, -0.254829592f));
+    const float2 neg_poly = __fmul2_rn(t, q);
+    const float2 s = __fmul2_rn(__fmul2_rn(ax, ax), make_float2(-kLog2e, -kLog2e));
+    e2 = make_float2(ex2_approx(s.x), ex2_approx(s.y));
+    const float2 r = __ffma2_rn(neg_poly, e2, make_float2(1.0f, 1.0f));
+    return __fadd2_rn(make_float2(1.0f, 1.0f), make_float2(copysignf(r.x, x.x), copysignf(r.y, x.y)));
 }
-// GELU and its derivative of a pair, erf and exponential shared: per lane the operations of gelu_f
-// and gelu_grad_f.
+// Two GELUs.  The forward epilogues and tvlbm_mlp_activation's g use it.
+__device__ __forceinline__ float2 gelu2_f(float2 z) {
+    float2 e2;
+    const float2 er1 = erf2_plus1(__fmul2_rn(z, make_float2(0.70710678118654752f, 0.70710678118654752f)), e2);
+    return __fmul2_rn(__fmul2_rn(make_float2(0.5f, 0.5f), z), er1);
+}
+// Two GELUs and their derivatives.
 __device__ __forceinline__ float2 gelu2_both(float2 z, float2& dg) {
-    const float2 x = __fmul2_rn(z, make_float2(0.70710678118654752f, 0.70710678118654752f));
-    const float2 ax = make_float2(fabsf(x.x), fabsf(x.y));
-    const float2 d = __ffma2_rn(make_float2(0.3275911f, 0.3275911f), ax, make_float2(1.0f, 1.0f));
-    const float2 t = make_float2(__fdividef(1.0f, d.x), __fdividef(1.0f, d.y));
-    float2 q = __ffma2_rn(t, make_float2(1.061405429f, 1.061405429f), make_float2(-1.453152027f, -1.453152027f));
-    q = __ffma2_rn(t, q, make_float2(1.421413741f, 1.421413741f));
-    q = __ffma2_rn(t, q, make_float2(-0.284496736f, -0.284496736f));
-    q = __ffma2_rn(t, q, make_float2(0.254829592f, 0.254829592f));
-    const float2 poly = __fmul2_rn(t, q);
-    const float2 sq = __fmul2_rn(make_float2(-ax.x, -ax.y), ax);
-    const float2 e2 = make_float2(__expf(sq.x), __expf(sq.y));
-    const float2 r = __ffma2_rn(make_float2(-poly.x, -poly.y), e2, make_float2(1.0f, 1.0f));
-    const float2 er1 = __fadd2_rn(make_float2(1.0f, 1.0f), make_float2(copysignf(r.x, x.x), copysignf(r.y, x.y)));
+    float2 e2;
     const float2 half = make_float2(0.5f, 0.5f);
+    const float2 er1 = erf2_plus1(__fmul2_rn(z, make_float2(0.70710678118654752f, 0.70710678118654752f)), e2);
     dg = __ffma2_rn(__fmul2_rn(z, make_float2(0.39894228040143268f, 0.39894228040143268f)), e2, __fmul2_rn(half, er1));
     return __fmul2_rn(__fmul2_rn(half, z), er1);
 }
@@ -131,14 +135,19 @@ __device__ __forceinline__ float warp_sum_f(float v) {
 
 // ---- fused inference: the three layers of one 128-row tile in one CTA ---------------------------
 // X, W1, W2, W3 arrive by TMA (128-byte swizzle); H1 and H2 never leave shared memory: the
-// epilogue threads write them in the same swizzled K-major layout the next MMA reads.  TMEM:
-// columns [0, 128) hold layer 1, [128, 256) layer 2, [0, 16) then layer 3.
+// epilogue threads write them in the same swizzled K-major layout the next MMA reads, over X and W1,
+// which layer 1 has consumed.  Every layer accumulates in the same 128 TMEM columns (its predecessor's
+// have been read by then).  69 KB and 40 registers: three CTAs per SM, so that two tiles' epilogues
+// run while a third waits for its products (65 536 rows of features: 21.4 us; 24.5 us with two CTAs, H
+// and a second accumulator of their own, and exponentials that handled subnormal results).  Launched
+// without programmatic overlap: blocks waiting for the kernel before take the room of its last ones
+// (the learned 256 x 256 step 33.9 instead of 32.0 us).
 struct FusedCfg {
-    static constexpr int X_OFF = 0, W1_OFF = 16384, W2_OFF = 32768, W3_OFF = 65536, H_OFF = 69632;
-    static constexpr int BYTES = H_OFF + 32768;  // 100 KB
+    static constexpr int X_OFF = 0, W1_OFF = 16384, W2_OFF = 32768, W3_OFF = 65536, H_OFF = 0;
+    static constexpr int BYTES = W3_OFF + 4096;
     static constexpr int SMEM = BYTES + 1024;
     static constexpr uint32_t TX = 16384 + 16384 + 32768 + 4096;
-    static constexpr uint32_t TMEM_COLS = 256;
+    static constexpr uint32_t TMEM_COLS = 128;
 };
 
 // Row r of a [128][128] BF16 tile stored as two 128-byte-swizzled K-major chunks of 64 columns:
@@ -181,7 +190,7 @@ __device__ __forceinline__ void feature_chunk(const MlpFeatures& f, int cell, fl
         }
         const int k = fi / 6, q = fi % 6;
         const int xx = k % 3 == 0 ? xm : (k % 3 == 1 ? cx : xp), yy = k / 3 == 0 ? ym : (k / 3 == 1 ? cy : yp);
-        v[e] = (__ldg(f.m6 + q * n + (long long)yy * f.nx + xx) - f.mu[q]) * f.isg[q];
+        v[e] = (*(f.m6 + q * n + (long long)yy * f.nx + xx) - f.mu[q]) * f.isg[q];
     }
 }
 
@@ -189,7 +198,7 @@ __device__ __forceinline__ void feature_chunk(const MlpFeatures& f, int cell, fl
 // instead of loaded by TMA; thread (row r, warpgroup g) makes features 16 g .. 16 g + 15 of row
 // r with the closure features kernel's arithmetic, so the inputs are the same BF16 values.
 template <bool FEAT>
-__global__ void __launch_bounds__(kFusedThreads) mlp_fused_forward_kernel(const __grid_constant__ CUtensorMap mx,
+__global__ void __launch_bounds__(kFusedThreads, 3) mlp_fused_forward_kernel(const __grid_constant__ CUtensorMap mx,
                                                                 const __grid_constant__ CUtensorMap mw1,
                                                                 const __grid_constant__ CUtensorMap mw2,
                                                                 const __grid_constant__ CUtensorMap mw3,
@@ -262,21 +271,27 @@ __global__ void __launch_bounds__(kFusedThreads) mlp_fused_forward_kernel(const 
     // layer 1 epilogue: H1 = g(Z1 + b1) into shared memory
     ok = __syncthreads_and((tid != 0 || ok) && bar_wait(&mma_bar, 0)) != 0;
     tc_fence_after();
-    if (ok) {
+    // a hidden layer's epilogue: this thread's columns, the biases four at a time
+    auto hidden = [&](const float* bias) {
 #pragma unroll 1
         for (int c0 = cbeg; c0 < cend; c0 += 16) {
             float v[16];
             __syncwarp();
             tmem_ld16(taddr + (uint32_t)c0, v);
 #pragma unroll
-            for (int k = 0; k < 16; k += 2) {
-                const float2 g = gelu2_f(__fadd2_rn(make_float2(v[k], v[k + 1]), make_float2(b1[c0 + k], b1[c0 + k + 1])));
-                v[k] = g.x;
-                v[k + 1] = g.y;
+            for (int k = 0; k < 16; k += 4) {
+                const float4 bk = *reinterpret_cast<const float4*>(bias + c0 + k);
+                const float2 g0 = gelu2_f(__fadd2_rn(make_float2(v[k], v[k + 1]), make_float2(bk.x, bk.y)));
+                const float2 g1 = gelu2_f(__fadd2_rn(make_float2(v[k + 2], v[k + 3]), make_float2(bk.z, bk.w)));
+                v[k] = g0.x;
+                v[k + 1] = g0.y;
+                v[k + 2] = g1.x;
+                v[k + 3] = g1.y;
             }
             store_h_sw128(hs, r, c0, v);
         }
-    }
+    };
+    if (ok) hidden(b1);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic writes -> MMA reads
     tc_fence_before();
     __syncthreads();
@@ -288,7 +303,7 @@ __global__ void __launch_bounds__(kFusedThreads) mlp_fused_forward_kernel(const 
             for (int kc = 0; kc < 2; ++kc)
 #pragma unroll
                 for (int kk = 0; kk < BK / 16; ++kk)
-                    mma_bf16(tmem + NH, sw128_desc(saddr(hs) + kc * 16384 + kk * 32),
+                    mma_bf16(tmem, sw128_desc(saddr(hs) + kc * 16384 + kk * 32),
                              sw128_desc(saddr(w2) + kc * 16384 + kk * 32), idesc, kc > 0 || kk > 0);
         }
         mma_commit(&mma_bar);
@@ -296,21 +311,7 @@ __global__ void __launch_bounds__(kFusedThreads) mlp_fused_forward_kernel(const 
     // layer 2 epilogue: H2 = g(Z2 + b2) over H1 (the MMA that read H1 has completed)
     ok = __syncthreads_and(ok && bar_wait(&mma_bar, 1)) != 0;
     tc_fence_after();
-    if (ok) {
-#pragma unroll 1
-        for (int c0 = cbeg; c0 < cend; c0 += 16) {
-            float v[16];
-            __syncwarp();
-            tmem_ld16(taddr + (uint32_t)(NH + c0), v);
-#pragma unroll
-            for (int k = 0; k < 16; k += 2) {
-                const float2 g = gelu2_f(__fadd2_rn(make_float2(v[k], v[k + 1]), make_float2(b2[c0 + k], b2[c0 + k + 1])));
-                v[k] = g.x;
-                v[k + 1] = g.y;
-            }
-            store_h_sw128(hs, r, c0, v);
-        }
-    }
+    if (ok) hidden(b2);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     tc_fence_before();
     __syncthreads();
@@ -338,7 +339,7 @@ __global__ void __launch_bounds__(kFusedThreads) mlp_fused_forward_kernel(const 
         for (int q = 0; q < 4; ++q) {
             float o[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) o[e] = 4 * q + e < NOUT ? v[4 * q + e] + b3[4 * q + e] : 0.0f;
+            for (int e = 0; e < 4; ++e) o[e] = 4 * q + e < NOUT ? v[4 * q + e] + __ldcg(b3 + 4 * q + e) : 0.0f;
             d[q] = make_float4(o[0], o[1], o[2], o[3]);
         }
     } else if (tid == 0 && status) {
@@ -369,10 +370,10 @@ __device__ __forceinline__ float column_sums32(float (&v)[32], int lane) {
 // dZ2, once the products that read them are done) and dY, all as 64-column chunks with 128-byte
 // rows.  TMEM (512 columns): the three weight gradients, accumulated over the CTA's tiles, Y, and
 // two 128-column work areas.  g'(Z) stays in registers between the passes (BF16, 16 per layer).
-// The products are tiny (0.14 MFLOP a row), so the chain of epilogues bounds it: 18 us for a tile, and
-// one CTA per SM runs up to 152 tiles in that time.  A batch of 4096 rows takes 28 us (with the
-// gradient reduction and Adam) where thirteen kernels, one product each with its operands and their
-// transposes through memory, took 155 us.
+// The products are tiny (0.14 MFLOP a row), so the chain of epilogues bounds it: 17 us for a tile, and
+// one CTA per SM runs up to 152 tiles in that time.  A batch of 4096 rows takes 27 us (with the
+// gradient reduction, 5.7 us, and Adam, 3.5) where thirteen kernels, one product each with its operands
+// and their transposes through memory, took 155 us.
 struct TrainCfg {
     static constexpr int X_OFF = 0, W1_OFF = 16384, W2_OFF = 32768, W3_OFF = 65536, H1_OFF = 69632, H2_OFF = 102400,
                          DY_OFF = 135168;
@@ -380,10 +381,17 @@ struct TrainCfg {
     static constexpr int SMEM = BYTES + 1024;
     static constexpr uint32_t TX_W = 16384 + 32768 + 4096, TX_X = 16384;
     static constexpr uint32_t T_DW2 = 0, T_DW1 = 128, T_DW3 = 192, T_Y = 208, T_A = 256, T_B = 384;
-    // a CTA's partial sums, floats: dW1 [128][64], dW2 [128][128], dW3 [16][128], then the bias
-    // gradients of the four 32-row groups: db1 [4][128], db2 [4][128], db3 [4][16]
-    static constexpr int P_W1 = 0, P_W2 = P_W1 + NH * NINP, P_W3 = P_W2 + NH * NH, P_B1 = P_W3 + NOUTP * NH,
-                         P_B2 = P_B1 + 4 * NH, P_B3 = P_B2 + 4 * NH, P_TOTAL = P_B3 + 4 * NOUTP;
+    // the second half tile's weight gradients (`halves`, below), in columns that are free by then
+    static constexpr uint32_t T_DW2H = T_A, T_DW1H = T_B, T_DW3H = 224;
+    // one partial sum of the weight gradients, floats, the hidden unit that owns a TMEM lane running fastest
+    // (so that a warp's stores are whole lines): dW1^T [64][128], dW2^T [128][128], dW3 [16][128]; and a
+    // CTA's bias gradients of its four 32-row groups: db1 [4][128], db2 [4][128], db3 [4][16]
+    static constexpr int P_W1 = 0, P_W2 = P_W1 + NH * NINP, P_W3 = P_W2 + NH * NH, P_SUM = P_W3 + NOUTP * NH;
+    static constexpr int P_B1 = 0, P_B2 = P_B1 + 4 * NH, P_B3 = P_B2 + 4 * NH, P_BIAS = P_B3 + 4 * NOUTP;
+    // Up to kHalfTiles tiles (8192 rows) every 64 rows give a partial sum of their own, beyond that every
+    // CTA's tiles one; the partial sums are added in row order.  (64-row sums added in FP32 are the
+    // summation that training runs have been reproduced with.)
+    static constexpr int kHalfTiles = 64;
 };
 
 // K = 16 slices kk of D (+)= A B^T over `steps` slices, operand starts ad / bd advancing by as / bs
@@ -399,9 +407,10 @@ __global__ void __launch_bounds__(kFusedThreads, 1) mlp_train_kernel(const __gri
                                                                      const __grid_constant__ CUtensorMap mw2,
                                                                      const __grid_constant__ CUtensorMap mw3,
                                                                      const float* __restrict__ theta,
-                                                                     const float* __restrict__ ystar, int tiles, float scale,
-                                                                     float* __restrict__ part, double* __restrict__ loss_part,
-                                                                     int* status) {
+                                                                     const float* __restrict__ ystar, int tiles, int halves,
+                                                                     float scale, float* __restrict__ part,
+                                                                     float* __restrict__ bias_part,
+                                                                     double* __restrict__ loss_part, int* status) {
     using Cfg = TrainCfg;
     static_assert(kFusedGroups == 4, "32 columns per thread and hidden layer");
     extern __shared__ unsigned char smem_raw[];
@@ -417,11 +426,13 @@ __global__ void __launch_bounds__(kFusedThreads, 1) mlp_train_kernel(const __gri
         bar_init(&mma_bar, 1);
         bar_init_fence();
     }
+    pdl_wait();  // the weights (and the partial sums' readers) of the kernels before this one
+    // TMEM only once the kernels before this one are complete: a block that held some while waiting for
+    // them could keep one of theirs from allocating
     if (warp == 0) tmem_alloc(&tmem_slot, 512);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    pdl_wait();  // the weights (and the partial sums' readers) of the kernels before this one
     const uint32_t tmem = tmem_slot;
     unsigned char *xs = base + Cfg::X_OFF, *w1 = base + Cfg::W1_OFF, *w2 = base + Cfg::W2_OFF, *w3 = base + Cfg::W3_OFF,
                   *h1 = base + Cfg::H1_OFF, *h2 = base + Cfg::H2_OFF, *dys = base + Cfg::DY_OFF;
@@ -460,6 +471,11 @@ __global__ void __launch_bounds__(kFusedThreads, 1) mlp_train_kernel(const __gri
         __syncthreads();
         tc_fence_after();
     };
+    // D (+)= A^T B over the tile's 128 rows; with halves (one tile per CTA) rows 64 .. 127 into Dh
+    auto rows_product = [&](uint32_t d, uint32_t dh, uint64_t a, uint64_t b, uint32_t idesc, bool accumulate) {
+        mma_chain(tmem + d, a, b, 128, 128, BM / 32, idesc, accumulate);
+        mma_chain(tmem + (halves ? dh : d), a + 128 * (BM / 32), b + 128 * (BM / 32), 128, 128, BM / 32, idesc, !halves);
+    };
     const uint32_t kk = idesc_bf16_f32(BM, NH), kk16 = idesc_bf16_f32(BM, NOUTP);
     constexpr uint32_t A_MN = 1u << 15, B_MN = 1u << 16;
     float db1 = 0.0f, db2 = 0.0f, db3 = 0.0f;  // column sums of this warp's rows: column cbeg + lane (db3: lane)
@@ -472,9 +488,14 @@ __global__ void __launch_bounds__(kFusedThreads, 1) mlp_train_kernel(const __gri
         const uint32_t xph = (uint32_t)((tile - (int)blockIdx.x) / (int)gridDim.x) & 1u;
         float4 ys[3];
         if (warp < 4) {  // the targets, long before they are needed
-            const float4* q = reinterpret_cast<const float4*>(ystar + (size_t)(m0 + r) * NOUTP);
+            const float* q = ystar + (size_t)(m0 + r) * NOUTP;
+            if ((reinterpret_cast<uintptr_t>(ystar) & 15) == 0) {
 #pragma unroll
-            for (int k = 0; k < 3; ++k) ys[k] = __ldg(q + k);
+                for (int k = 0; k < 3; ++k) ys[k] = __ldg(reinterpret_cast<const float4*>(q) + k);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 3; ++k) ys[k] = make_float4(q[4 * k], q[4 * k + 1], q[4 * k + 2], q[4 * k + 3]);
+            }
         }
         if (tid == 0) {
             ok = (!first || bar_wait(&w_bar, 0)) && bar_wait(&x_bar, xph);
@@ -553,8 +574,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) mlp_train_kernel(const __gri
             if (ok) {
                 // dH2 = dY W3 (contracts the 16 outputs), dW3^T += H2^T dY (contracts the rows)
                 mma_chain(tmem + Cfg::T_A, sw128_desc(saddr(dys)), sw128_mn_desc(saddr(w3), 2048), 0, 0, 1, kk | B_MN, false);
-                mma_chain(tmem + Cfg::T_DW3, sw128_mn_desc(saddr(h2), 16384), sw128_mn_desc(saddr(dys), 16384), 128, 128,
-                          BM / 16, kk16 | A_MN | B_MN, !first);
+                rows_product(Cfg::T_DW3, Cfg::T_DW3H, sw128_mn_desc(saddr(h2), 16384), sw128_mn_desc(saddr(dys), 16384),
+                             kk16 | A_MN | B_MN, !first);
             }
             mma_commit(&mma_bar);
         }
@@ -588,8 +609,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) mlp_train_kernel(const __gri
                 for (int kc = 0; kc < 2; ++kc)
                     mma_chain(tmem + Cfg::T_B, sw128_desc(saddr(h2) + kc * 16384),
                               sw128_mn_desc(saddr(w2) + kc * 8192, 16384), 2, 128, BK / 16, kk | B_MN, kc > 0);
-                mma_chain(tmem + Cfg::T_DW2, sw128_mn_desc(saddr(h2), 16384), sw128_mn_desc(saddr(h1), 16384), 128, 128,
-                          BM / 16, kk | A_MN | B_MN, !first);
+                rows_product(Cfg::T_DW2, Cfg::T_DW2H, sw128_mn_desc(saddr(h2), 16384), sw128_mn_desc(saddr(h1), 16384),
+                             kk | A_MN | B_MN, !first);
             }
             mma_commit(&mma_bar);
         }
@@ -598,8 +619,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) mlp_train_kernel(const __gri
         operands_ready();
         if (tid == 0) {
             if (ok)  // dW1 += dZ1^T X
-                mma_chain(tmem + Cfg::T_DW1, sw128_mn_desc(saddr(h1), 16384), sw128_mn_desc(saddr(xs), 16384), 128, 128,
-                          BM / 16, idesc_bf16_f32(BM, NINP) | A_MN | B_MN, !first);
+                rows_product(Cfg::T_DW1, Cfg::T_DW1H, sw128_mn_desc(saddr(h1), 16384), sw128_mn_desc(saddr(xs), 16384),
+                             idesc_bf16_f32(BM, NINP) | A_MN | B_MN, !first);
             mma_commit(&mma_bar);
         }
         products_done();
@@ -610,28 +631,29 @@ __global__ void __launch_bounds__(kFusedThreads, 1) mlp_train_kernel(const __gri
     }
 
     if (ok) {
-        float* q = part + (size_t)blockIdx.x * Cfg::P_TOTAL;
         float v[16];
-        auto drain = [&](uint32_t t0, float* row) {
+        auto drain = [&](uint32_t t0, float* q) {  // 16 columns of this thread's lane
             __syncwarp();
             tmem_ld16(taddr + t0, v);
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                reinterpret_cast<float4*>(row)[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+            for (int k = 0; k < 16; ++k) q[k * NH + r] = v[k];
         };
-        drain(Cfg::T_DW2 + cbeg, q + Cfg::P_W2 + r * NH + cbeg);
-        drain(Cfg::T_DW2 + cbeg + 16, q + Cfg::P_W2 + r * NH + cbeg + 16);
-        drain(Cfg::T_DW1 + cbeg / 2, q + Cfg::P_W1 + r * NINP + cbeg / 2);
+        auto sums_out = [&](float* q, uint32_t dw1, uint32_t dw2, uint32_t dw3) {
+            drain(dw2 + cbeg, q + Cfg::P_W2 + cbeg * NH);
+            drain(dw2 + cbeg + 16, q + Cfg::P_W2 + (cbeg + 16) * NH);
+            drain(dw1 + cbeg / 2, q + Cfg::P_W1 + cbeg / 2 * NH);
+            if (warp < 4) drain(dw3, q + Cfg::P_W3);
+        };
+        float* q = part + (size_t)blockIdx.x * (halves ? 2 : 1) * Cfg::P_SUM;
+        sums_out(q, Cfg::T_DW1, Cfg::T_DW2, Cfg::T_DW3);
+        if (halves) sums_out(q + Cfg::P_SUM, Cfg::T_DW1H, Cfg::T_DW2H, Cfg::T_DW3H);
+        float* qb = bias_part + (size_t)blockIdx.x * Cfg::P_BIAS;
         if (warp < 4) {
-            __syncwarp();
-            tmem_ld16(taddr + Cfg::T_DW3, v);
-#pragma unroll
-            for (int k = 0; k < NOUTP; ++k) q[Cfg::P_W3 + k * NH + r] = v[k];
-            if (lane < NOUTP) q[Cfg::P_B3 + warp * NOUTP + lane] = db3;
+            if (lane < NOUTP) qb[Cfg::P_B3 + warp * NOUTP + lane] = db3;
             if (lane == 0) loss_part[blockIdx.x * 4 + warp] = loss;
         }
-        q[Cfg::P_B1 + (warp & 3) * NH + cbeg + lane] = db1;
-        q[Cfg::P_B2 + (warp & 3) * NH + cbeg + lane] = db2;
+        qb[Cfg::P_B1 + (warp & 3) * NH + cbeg + lane] = db1;
+        qb[Cfg::P_B2 + (warp & 3) * NH + cbeg + lane] = db2;
     } else if (tid == 0) {
         if (status) atomicOr(status, 1);
         // let the loads started so far land before the CTA exits (bounded)
@@ -645,16 +667,15 @@ __global__ void __launch_bounds__(kFusedThreads, 1) mlp_train_kernel(const __gri
 
 // ---- small kernels ---------------------------------------------------------------------------
 
-// grad[i] = the CTAs' partial sums in a fixed order: 64 parameters per block, four threads each
-// taking every fourth CTA; the last block sums the loss.
-__global__ void __launch_bounds__(256) reduce_gradient_kernel(const float* __restrict__ part,
-                                                              const double* __restrict__ loss_part, int ctas,
-                                                              float* __restrict__ grad, double* __restrict__ loss) {
+// The gradient: a weight's `sums` partial sums in row order, a bias's sums over the CTAs' row groups;
+// one thread per weight, 64 per block so that the blocks spread over the SMs.  The last block sums
+// the loss.
+__global__ void __launch_bounds__(64) reduce_gradient_kernel(const float* __restrict__ part, const float* __restrict__ bias_part,
+                                                             const double* __restrict__ loss_part, int sums, int ctas,
+                                                             float* __restrict__ grad, double* __restrict__ loss) {
     using Cfg = TrainCfg;
-    __shared__ float sh[4][64];
     pdl_launch_dependents();
     pdl_wait();
-    const int t = threadIdx.x & 63, g = threadIdx.x >> 6;
     if (blockIdx.x == gridDim.x - 1) {
         if (threadIdx.x < 32) {
             double l = 0.0;
@@ -665,25 +686,47 @@ __global__ void __launch_bounds__(256) reduce_gradient_kernel(const float* __res
         }
         return;
     }
-    const int i = blockIdx.x * 64 + t;
-    int off = 0, groups = 1, ld = 0;
-    if (i < OFF_B1) off = Cfg::P_W1 + (i / NIN) * NINP + i % NIN;
-    else if (i < OFF_W2) off = Cfg::P_B1 + i - OFF_B1, groups = 4, ld = NH;
-    else if (i < OFF_B2) off = Cfg::P_W2 + i - OFF_W2;
-    else if (i < OFF_W3) off = Cfg::P_B2 + i - OFF_B2, groups = 4, ld = NH;
-    else if (i < OFF_B3) off = Cfg::P_W3 + i - OFF_W3;
-    else off = Cfg::P_B3 + i - OFF_B3, groups = 4, ld = NOUTP;
-    float acc = 0.0f;
-    if (i < NPARAM) {
-#pragma unroll 8
-        for (int c = g; c < ctas; c += 4) acc += __ldcg(part + (size_t)c * Cfg::P_TOTAL + off);
-        for (int k = 1; k < groups; ++k)
-            for (int c = g; c < ctas; c += 4) acc += __ldcg(part + (size_t)c * Cfg::P_TOTAL + off + k * ld);
+    // (a warp reads one line per partial sum; blocks beyond the weights' take the biases)
+    const int t = blockIdx.x * 64 + threadIdx.x;
+    if (t < Cfg::P_SUM) {
+        float acc = 0.0f;
+#pragma unroll 16
+        for (int c = 0; c < sums; ++c) acc += __ldcg(part + (size_t)c * Cfg::P_SUM + t);
+        if (t < Cfg::P_W2) {
+            const int c = t / NH, r = t % NH;
+            if (c < NIN) grad[OFF_W1 + r * NIN + c] = acc;
+        } else if (t < Cfg::P_W3) {
+            const int c = (t - Cfg::P_W2) / NH, r = (t - Cfg::P_W2) % NH;
+            grad[OFF_W2 + r * NH + c] = acc;
+        } else if (t - Cfg::P_W3 < NOUT * NH) {
+            grad[OFF_W3 + t - Cfg::P_W3] = acc;
+        }
+        return;
     }
-    sh[g][t] = acc;
-    __syncthreads();
-    if (g == 0 && i < NPARAM) grad[i] = (sh[0][t] + sh[1][t]) + (sh[2][t] + sh[3][t]);
+    // a bias per warp, its lanes sharing the CTAs' row groups, in compensated FP32 (each addition's
+    // rounding error is kept by the two-sum identity; FP64 would take 64 cycles a warp instruction)
+    const int k = (t - Cfg::P_SUM) >> 5, lane = threadIdx.x & 31;  // b1, b2, b3
+    if (k >= 2 * NH + NOUT) return;
+    const int boff = k < NH ? Cfg::P_B1 + k : k < 2 * NH ? Cfg::P_B2 + k - NH : Cfg::P_B3 + k - 2 * NH;
+    const int ld = k < 2 * NH ? NH : NOUTP;
+    float a = 0.0f, err = 0.0f;
+    const auto add = [&](float v) {
+        const float sum = __fadd_rn(a, v), av = __fadd_rn(sum, -a);
+        err = __fadd_rn(err, __fadd_rn(__fadd_rn(a, -__fadd_rn(sum, -av)), __fadd_rn(v, -av)));
+        a = sum;
+    };
+#pragma unroll 4
+    for (int c = lane; c < 4 * ctas; c += 32) add(__ldcg(bias_part + (size_t)(c >> 2) * Cfg::P_BIAS + boff + (c & 3) * ld));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float other = __shfl_down_sync(0xffffffffu, a, o);
+        err = __fadd_rn(err, __shfl_down_sync(0xffffffffu, err, o));
+        add(other);
+    }
+    if (lane == 0) grad[k < NH ? OFF_B1 + k : k < 2 * NH ? OFF_B2 + k - NH : OFF_B3 + k - 2 * NH] = __fadd_rn(a, err);
 }
+constexpr int kReduceBlocks = TrainCfg::P_SUM / 64 + (2 * NH + NOUT + 1) / 2 + 1;
+static_assert(TrainCfg::P_SUM % 64 == 0, "whole blocks of weights");
 
 // The BF16 copy of parameter i in the layout the products read (zero padding where K or N is padded:
 // written once, when the network is created).
@@ -728,12 +771,12 @@ struct tvlbm_mlp {
     cudaStream_t stream;
     unsigned char* mem;
     size_t bytes;
-    float *theta, *m1, *m2, *grad, *part;
+    float *theta, *m1, *m2, *grad, *part, *bias_part;
     double *loss, *loss_part;
     int* status;
     bf16 *w1p, *w2, *w3p;
     float* ybuf;
-    int ctas;  // most CTAs of a training pass (one per SM), the partial sums' extent
+    int ctas;  // most CTAs of a training pass (one per SM)
     int adam_t;
     unsigned long long uid;
     // descriptors of the last inference call (inputs at cached_x, cached_rows rows)
@@ -830,9 +873,9 @@ int mlp_forward_async(tvlbm_mlp* m, const void* x, int rows, float* y) {
     }
     MlpFeatures none;
     memset(&none, 0, sizeof(none));
-    mlp_fused_forward_kernel<false><<<tiles, kFusedThreads, FusedCfg::SMEM, m->stream>>>(mx, mw1, mw2, mw3, m->theta, y,
-                                                                                        m->status, none);
-    MLP_CUDA(m, cudaGetLastError(), "fused forward");
+    MLP_CUDA(m, launch_as(false, mlp_fused_forward_kernel<false>, dim3(tiles), dim3(kFusedThreads), FusedCfg::SMEM, m->stream, mx,
+                           mw1, mw2, mw3, (const float*)m->theta, y, m->status, none),
+             "fused forward");
     return TVLBM_OK;
 }
 
@@ -857,9 +900,9 @@ int mlp_forward_features_async(tvlbm_mlp* m, const MlpFeatures& feat, int rows, 
                  "fused forward attribute");
         attr_set[dev] = true;
     }
-    mlp_fused_forward_kernel<true><<<tiles, kFusedThreads, FusedCfg::SMEM, m->stream>>>(mx, mw1, mw2, mw3, m->theta, y,
-                                                                                       m->status, feat);
-    MLP_CUDA(m, cudaGetLastError(), "fused forward with features");
+    MLP_CUDA(m, launch_as(false, mlp_fused_forward_kernel<true>, dim3(tiles), dim3(kFusedThreads), FusedCfg::SMEM, m->stream, mx,
+                           mw1, mw2, mw3, (const float*)m->theta, y, m->status, feat),
+             "fused forward with features");
     return TVLBM_OK;
 }
 int mlp_max_rows(const tvlbm_mlp* m) { return m->max_rows; }
@@ -899,8 +942,10 @@ int tvlbm_mlp_create(int max_rows, tvlbm_mlp** out) {
         return o;
     };
     const size_t o_theta = take(NPARAM * 4), o_m1 = take(NPARAM * 4), o_m2 = take(NPARAM * 4), o_grad = take(NPARAM * 4);
-    const size_t o_part = take((size_t)m->ctas * TrainCfg::P_TOTAL * 4), o_losses = take((size_t)m->ctas * 4 * 8),
-                 o_loss = take(8), o_status = take(4);
+    const int half_tiles = max_rows / BM < TrainCfg::kHalfTiles ? max_rows / BM : TrainCfg::kHalfTiles;
+    const size_t sums = m->ctas > 2 * half_tiles ? m->ctas : 2 * half_tiles;  // partial sums of a pass
+    const size_t o_part = take(sums * TrainCfg::P_SUM * 4), o_bias = take((size_t)m->ctas * TrainCfg::P_BIAS * 4),
+                 o_losses = take((size_t)m->ctas * 4 * 8), o_loss = take(8), o_status = take(4);
     const size_t o_y = take(R * NOUTP * 4);
     const size_t o_w1p = take(NH * NINP * 2), o_w2 = take(NH * NH * 2), o_w3p = take(NOUTP * NH * 2);
     m->bytes = off;
@@ -917,6 +962,7 @@ int tvlbm_mlp_create(int max_rows, tvlbm_mlp** out) {
     m->loss = (double*)(b + o_loss);
     m->status = (int*)(b + o_status);
     m->ybuf = (float*)(b + o_y);
+    m->bias_part = (float*)(b + o_bias);
     m->loss_part = (double*)(b + o_losses);
     m->w1p = (bf16*)(b + o_w1p);
     m->w2 = (bf16*)(b + o_w2);
@@ -982,11 +1028,11 @@ int tvlbm_mlp_loss_grad(tvlbm_mlp* m, const void* x, const float* ystar, int row
     cudaSetDevice(m->device);
     cudaStream_t s = m->stream;
     const int tiles = rows / BM, ctas = tiles < m->ctas ? tiles : m->ctas;
+    const int halves = tiles <= TrainCfg::kHalfTiles && tiles <= m->ctas ? 1 : 0;  // (one tile per CTA)
     CUtensorMap mx, mw1, mw2, mw3;
     if (!bf16_map(&mx, x, NINP, rows, NINP, BM) || !bf16_map(&mw1, m->w1p, NINP, NH, NINP, NH) ||
         !bf16_map(&mw2, m->w2, NH, NH, NH, NH) || !bf16_map(&mw3, m->w3p, NH, NOUTP, NH, NOUTP))
         return mfail(m, TVLBM_EINVAL, "TMA descriptor rejected (alignment of x?)");
-    if ((uintptr_t)ystar & 15) return mfail(m, TVLBM_EINVAL, "ystar must be 16-byte aligned");
     static bool attr_set[64] = {};
     if (m->device < 0 || m->device >= 64 || !attr_set[m->device]) {
         MLP_CUDA(m, cudaFuncSetAttribute(mlp_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TrainCfg::SMEM),
@@ -994,11 +1040,12 @@ int tvlbm_mlp_loss_grad(tvlbm_mlp* m, const void* x, const float* ystar, int row
         if (m->device >= 0 && m->device < 64) attr_set[m->device] = true;
     }
     MLP_CUDA(m, launch_pdl(mlp_train_kernel, dim3(ctas), dim3(kFusedThreads), TrainCfg::SMEM, s, mx, mw1, mw2, mw3,
-                           (const float*)m->theta, ystar, tiles, 2.0f / ((float)rows * (float)NOUT), m->part, m->loss_part,
-                           m->status),
+                           (const float*)m->theta, ystar, tiles, halves, 2.0f / ((float)rows * (float)NOUT), m->part,
+                           m->bias_part, m->loss_part, m->status),
              "training pass");
-    MLP_CUDA(m, launch_pdl(reduce_gradient_kernel, dim3((NPARAM + 63) / 64 + 1), dim3(256), 0, s, (const float*)m->part,
-                           (const double*)m->loss_part, ctas, m->grad, m->loss),
+    MLP_CUDA(m, launch_pdl(reduce_gradient_kernel, dim3(kReduceBlocks), dim3(64), 0, s, (const float*)m->part,
+                           (const float*)m->bias_part, (const double*)m->loss_part, halves ? 2 * tiles : ctas, ctas, m->grad,
+                           m->loss),
              "gradient reduction");
     if (loss || grad) {
         double l = 0.0;
