@@ -613,22 +613,27 @@ __device__ __forceinline__ void fence_acquire_gpu() { asm volatile("fence.acq_re
 __device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 
 // Task sources of the dataflow kernel.  flow_task(): the step k and tile t of task number `task` and
-// the completion counters of t's 3 x 3 periodic neighbourhood; flow_tile(): where tile t is, its
-// domain's geometry, the descriptors it loads its step-k windows with and stores its step-k output
-// with, and the buffer its periodic images go to.
+// the completion counter of neighbour d (0 .. 8) of t's 3 x 3 periodic neighbourhood; flow_tile(): where
+// tile t is, its domain's geometry, the descriptors it loads its step-k windows with and stores its
+// step-k output with, and the buffer its periodic images go to.
+// Tile (tx + d % 3 - 1, ty + d / 3 - 1) of a tiles_x x tiles_y grid, wrapped (by comparison: a division
+// is about 25 instructions).
+__device__ __forceinline__ int flow_neighbour(int tx, int ty, int d, int tiles_x, int tiles_y) {
+    const int dy = d >= 6 ? 1 : (d >= 3 ? 0 : -1), dx = d - 3 * (dy + 1) - 1;
+    int xx = tx + dx, yy = ty + dy;
+    xx = xx < 0 ? xx + tiles_x : (xx >= tiles_x ? xx - tiles_x : xx);
+    yy = yy < 0 ? yy + tiles_y : (yy >= tiles_y ? yy - tiles_y : yy);
+    return yy * tiles_x + xx;
+}
 // One domain (FlowSrc, see tvlbm_kernels.cuh): step k visits tile rows starting at row k (the
 // first rows of step k + 1 then depend on the first rows that step k finished).
-__device__ __forceinline__ void flow_task(const FlowSrc& src, int task, int& k, int& t, const int* (&nb)[9]) {
+__device__ __forceinline__ void flow_task(const FlowSrc& src, int task, int d, int& k, int& t, const int*& nb) {
     k = task / src.ntiles;
     const int r = task - k * src.ntiles;
-    const int tx = r % src.tiles_x, ty = (r / src.tiles_x + k) % src.tiles_y;
+    const int ry = r / src.tiles_x, tx = r - ry * src.tiles_x;
+    const int ty = (ry + k) % src.tiles_y;
     t = ty * src.tiles_x + tx;
-#pragma unroll
-    for (int d = 0; d < 9; ++d) {
-        const int xx = (tx + d % 3 - 1 + src.tiles_x) % src.tiles_x;
-        const int yy = (ty + d / 3 - 1 + src.tiles_y) % src.tiles_y;
-        nb[d] = src.done + yy * src.tiles_x + xx;
-    }
+    nb = src.done + flow_neighbour(tx, ty, d, src.tiles_x, src.tiles_y);
 }
 __device__ __forceinline__ void flow_tile(const FlowSrc& src, int t, int k, const KParams& p, int TX, int TY, int& x0,
                                           int& y0, Geom& g, const CUtensorMap*& lmap, const CUtensorMap*& smap,
@@ -658,18 +663,13 @@ struct BatchFlowSrc {
     long long wait_ns;
     int wait_extra;
 };
-__device__ __forceinline__ void flow_task(const BatchFlowSrc& src, int task, int& k, int& t, const int* (&nb)[9]) {
+__device__ __forceinline__ void flow_task(const BatchFlowSrc& src, int task, int d, int& k, int& t, const int*& nb) {
     k = task / src.ntiles;
     t = task - k * src.ntiles;
     const BatchDomain& D = src.dom[__ldg(src.tile_dom + t)];
     const int local = t - D.tile_begin;
-    const int tx = local % D.tiles_x, ty = local / D.tiles_x;
-#pragma unroll
-    for (int d = 0; d < 9; ++d) {
-        const int xx = (tx + d % 3 - 1 + D.tiles_x) % D.tiles_x;
-        const int yy = (ty + d / 3 - 1 + D.tiles_y) % D.tiles_y;
-        nb[d] = src.done + D.tile_begin + yy * D.tiles_x + xx;
-    }
+    const int ty = local / D.tiles_x, tx = local - ty * D.tiles_x;
+    nb = src.done + D.tile_begin + flow_neighbour(tx, ty, d, D.tiles_x, D.tiles_y);
 }
 __device__ __forceinline__ void flow_tile(const BatchFlowSrc& src, int t, int k, const KParams& p, int TX, int TY,
                                           int& x0, int& y0, Geom& g, const CUtensorMap*& lmap,
@@ -734,7 +734,7 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 
-// Producer (lane 0 of the first extra warp): take a task, wait for its neighbourhood, wait for a
+// Producer (the first extra warp): take a task, wait for its neighbourhood, wait for a
 // free stage, publish the task in the stage's slot and start its Q window loads.  A negative slot
 // value ends the consumers' loop (-1: no tasks left, -2: a wait gave up).  Consumers (the tiled
 // form's threads): wait for a stage, compute the tile, free the stage, and publish the tile's
@@ -804,7 +804,9 @@ __global__ void __launch_bounds__(FlowCfg<N1, C, CFG>::THREADS, FlowCfg<N1, C, C
     }
 
     if (tid >= F::CONSUMERS) {  // ---- producer warp ----
-        if (tid != F::CONSUMERS) return;
+        // The whole warp works on every task: one neighbour's counter per lane, one window load per
+        // lane (a single thread took 3.4 us per task, 95 % of the 24 us per step at 1024 x 1024).
+        const int lane = tid - F::CONSUMERS;
         // Issue the TMA loads of task `task` (step k, tile t) into stage st and publish it.
         auto issue = [&](int st, int t, int k) {
             int x0, y0;
@@ -812,84 +814,84 @@ __global__ void __launch_bounds__(FlowCfg<N1, C, CFG>::THREADS, FlowCfg<N1, C, C
             const CUtensorMap *map, *smap;
             void* outp;
             flow_tile(src, t, k, p, TX, TY, x0, y0, g, map, smap, outp);
-            slot[st] = t;  // slots: [stage] tile (>= 0) or end code, [STAGES + stage] step
-            slot[F::STAGES + st] = k;
-            mbar_arrive_expect_tx(&full[st], F::TX_BYTES);
+            if (lane == 0) {
+                slot[st] = t;  // slots: [stage] tile (>= 0) or end code, [STAGES + stage] step
+                slot[F::STAGES + st] = k;
+                mbar_arrive_expect_tx(&full[st], F::TX_BYTES);
+            }
+            __syncwarp();
             unsigned char* sb = base + st * F::STAGE_BYTES;
+            static_assert(Q <= 64, "two windows per lane");
 #pragma unroll
-            for (int l = 0; l < Q; ++l) {
-                const int i = l % N1, j = l / N1;
-                tma_load_3d(sb + l * WIN, map, &full[st], (x0 + g.hx - p.sh[i] - 1) & ~(A - 1), y0 + HY - p.sh[j] - 1,
-                            l);
+            for (int h = 0; h < (Q + 31) / 32; ++h) {
+                const int l = lane + 32 * h;
+                if (l < Q) {
+                    const int i = l % N1, j = l / N1;
+                    tma_load_3d(sb + l * WIN, map, &full[st], (x0 + g.hx - p.sh[i] - 1) & ~(A - 1), y0 + HY - p.sh[j] - 1,
+                                l);
+                }
             }
         };
-        // Wait (bounded) until the 3 x 3 neighbourhoods of nt tasks (their completion counters nb,
-        // the counts need) have completed their previous step: 0, or -2 once the wait gives up.
-        auto await_nb = [&](const int* const (*nb)[9], const int* need, int nt) -> int {
+        // Wait (bounded) until every lane's counter nb has reached the count need (need < 0: none to
+        // wait for), then order the loads that follow behind what the counters published: 0, or -2 once
+        // the wait gives up.
+        auto await_nb = [&](const int* nb, int need) -> int {
             const uint64_t t0 = global_ns();
             for (;;) {
-                int ready = 0;
-                for (int q = 0; q < nt; ++q)
-#pragma unroll
-                    for (int d = 0; d < 9; ++d) ready += ld_relaxed_gpu(nb[q][d]) >= need[q] ? 1 : 0;
-                if (ready == 9 * nt) return 0;
-                if (*(volatile int*)src.abort || global_ns() - t0 > (uint64_t)src.wait_ns) return -2;
-                __nanosleep(64);
+                const bool ready = need < 0 || ld_relaxed_gpu(nb) >= need;
+                if (__all_sync(0xffffffffu, ready)) break;
+                const bool stop = *(volatile int*)src.abort || global_ns() - t0 > (uint64_t)src.wait_ns;
+                if (__any_sync(0xffffffffu, stop)) return -2;
+                __nanosleep(32);
             }
+            fence_acquire_gpu();
+            __syncwarp();  // every lane's acquired counters before any lane's loads
+            fence_proxy_async_global();
+            return 0;
         };
         // Tasks come two at a time (stage 0, then stage 1, in the order they were handed out).
         // Two tasks of the same step do not depend on each other: their neighbourhoods are polled
-        // together and one acquire fence covers both (the fence is the larger part of a task's
-        // cost for this thread).  Across a step boundary the second may depend on the first, so
-        // it is polled only after the first is issued.  With one stage, one task at a time.
+        // together (lanes 0 .. 8 and 9 .. 17) and one acquire fence covers both (the fence is the larger
+        // part of a task's cost for this warp).  Across a step boundary the second may depend on the
+        // first, so it is polled only after the first is issued.  With one stage, one task at a time.
         constexpr int PAIR = F::STAGES == 2 ? 2 : 1;
+        const int mine = lane / 9, d = lane - 9 * mine;  // this lane's task of the pair, its neighbour
         for (int m = 0;; ++m) {
-            const int task0 = atomicAdd(src.next_task, PAIR);
+            int task0 = 0;
+            if (lane == 0) task0 = atomicAdd(src.next_task, PAIR);
+            task0 = __shfl_sync(0xffffffffu, task0, 0);
             const bool together = PAIR == 2 && task0 / src.ntiles == (task0 + 1) / src.ntiles;
-            int code[2], k[2] = {0, 0}, t[2] = {0, 0}, need[2] = {0, 0};
-            const int* nb[2][9];
-            int nt = 0;  // tasks of this round that exist
-#pragma unroll
-            for (int q = 0; q < PAIR; ++q) {
-                code[q] = task0 + q < total ? 0 : -1;
-                if (!code[q]) {
-                    flow_task(src, task0 + q, k[q], t[q], nb[q]);
-                    need[q] = k[q] * F::DONE_PER_TASK + src.wait_extra;
-                    ++nt;
-                }
-            }
-            bool fenced = false;
-            if (together && nt > 0) {
-                const int c = await_nb(nb, need, nt);
-                if (c) code[0] = code[1] = c;
-                else {
-                    fence_acquire_gpu();
-                    fence_proxy_async_global();
-                    fenced = true;
-                }
-            }
+            // step and tile of this lane's task (lanes 18 .. 31: of the second, unused)
+            const int q0 = PAIR == 2 && mine ? 1 : 0;
+            const bool exists = task0 + q0 < total;
+            int k = 0, t = 0;
+            const int* nb = src.done;
+            if (exists) flow_task(src, task0 + q0, d < 9 && mine < 2 ? d : 4, k, t, nb);
+            const int need = exists && mine < PAIR ? k * F::DONE_PER_TASK + src.wait_extra : -1;
+            const int k1 = __shfl_sync(0xffffffffu, k, 9), t1 = __shfl_sync(0xffffffffu, t, 9);
+            const int k0 = __shfl_sync(0xffffffffu, k, 0), t0 = __shfl_sync(0xffffffffu, t, 0);
+            int early = 1;  // result of polling both together (1: not polled yet)
+            if (together && task0 < total) early = await_nb(nb, need);
 #pragma unroll
             for (int q = 0; q < PAIR; ++q) {
                 const int st = q, n = PAIR * m + q;
                 const uint32_t par = ((n / F::STAGES) & 1) ^ 1;  // first use of each stage passes at once
-                if (!code[q] && !fenced) {
-                    code[q] = await_nb(nb + q, need + q, 1);
-                    if (!code[q]) {
-                        fence_acquire_gpu();
-                        fence_proxy_async_global();
+                int code = task0 + q < total ? 0 : -1;
+                if (!code) code = early <= 0 ? early : await_nb(nb, mine == q ? need : -1);
+                const bool free_ok = __all_sync(0xffffffffu, mbar_wait_bounded(&empty[st], par, kWaitLimitNs));
+                if (!free_ok) code = -2;
+                if (code) {
+                    if (lane == 0) {
+                        if (code == -2) {
+                            atomicExch(src.abort, 1);
+                            if (p.status) atomicOr(p.status, 1);
+                        }
+                        slot[st] = code;
+                        mbar_arrive(&full[st]);  // release: the consumers see the slot
                     }
-                }
-                if (!mbar_wait_bounded(&empty[st], par, kWaitLimitNs)) code[q] = -2;
-                if (code[q] == -2) {
-                    atomicExch(src.abort, 1);
-                    if (p.status) atomicOr(p.status, 1);
-                }
-                if (code[q]) {
-                    slot[st] = code[q];
-                    mbar_arrive(&full[st]);  // release: the consumers see the slot
                     return;
                 }
-                issue(st, t[q], k[q]);
+                issue(st, q ? t1 : t0, q ? k1 : k0);
             }
         }
     }
