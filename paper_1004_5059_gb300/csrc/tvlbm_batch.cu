@@ -113,7 +113,7 @@ bool make_batch_layout(std::vector<DomainHost>& dom, int Q, int storage, BatchLa
     B->maps_off = B->tables_off + B->dom_bytes;
     B->maps_bytes = align_up(dom.size() * 2 * sizeof(CUtensorMap), 256);
     B->tiles_off = B->maps_off + B->maps_bytes;
-    B->tiles_bytes = align_up((size_t)max_tiles * sizeof(int), 256);
+    B->tiles_bytes = align_up((size_t)max_tiles * sizeof(BatchTile), 256);
     B->smaps_off = B->tiles_off + B->tiles_bytes;
     B->flow_off = B->smaps_off + B->maps_bytes;
     B->flow_bytes = align_up(((size_t)kFlowDone + max_tiles) * sizeof(int), 256);
@@ -147,7 +147,7 @@ int upload_tables(tvlbm_batch* b) {
     const size_t es = elem_size(b->storage);
     std::vector<BatchDomain> tab(b->count);
     std::vector<CUtensorMap> maps(2 * b->count), smaps(2 * b->count);
-    std::vector<int> tiles;
+    std::vector<BatchTile> tiles;
     tiles.reserve(b->B.max_tiles);
     for (int d = 0; d < b->count; ++d) {
         const DomainHost& D = b->dom[d];
@@ -165,7 +165,7 @@ int upload_tables(tvlbm_batch* b) {
         T.omegad = b->dt / D.tau;
         T.omegaf = (float)T.omegad;
         const int nt = T.tiles_x * ((D.ny + ty - 1) / ty);
-        for (int k = 0; k < nt; ++k) tiles.push_back(d);
+        for (int k = 0; k < nt; ++k) tiles.push_back({k % T.tiles_x * tx, k / T.tiles_x * ty, d, 0});
         for (int w = 0; w < 2; ++w)
             if (!encode_tensor_map(&maps[2 * d + w], dom_buf(b, d, w), b->storage, D.L, b->Q, bx, by) ||
                 !encode_tensor_map(&smaps[2 * d + w], dom_buf(b, d, w), b->storage, D.L, b->Q, tx, ty))
@@ -178,7 +178,7 @@ int upload_tables(tvlbm_batch* b) {
                              cudaMemcpyHostToDevice, b->stream), "upload descriptors");
     BCUDA(b, cudaMemcpyAsync(bptr(b, b->B.smaps_off), smaps.data(), smaps.size() * sizeof(CUtensorMap),
                              cudaMemcpyHostToDevice, b->stream), "upload descriptors");
-    BCUDA(b, cudaMemcpyAsync(bptr(b, b->B.tiles_off), tiles.data(), tiles.size() * sizeof(int),
+    BCUDA(b, cudaMemcpyAsync(bptr(b, b->B.tiles_off), tiles.data(), tiles.size() * sizeof(BatchTile),
                              cudaMemcpyHostToDevice, b->stream), "upload tile list");
     BCUDA(b, cudaStreamSynchronize(b->stream), "table upload synchronize");
     return TVLBM_OK;
@@ -221,7 +221,7 @@ cudaError_t launch_batch_flow(tvlbm_batch* b, int n, int parity, cudaStream_t s)
         src.dom = (const BatchDomain*)bptr(b, b->B.tables_off);
         src.lmaps = (const CUtensorMap*)bptr(b, b->B.maps_off);
         src.smaps = (const CUtensorMap*)bptr(b, b->B.smaps_off);
-        src.tile_dom = (const int*)bptr(b, b->B.tiles_off);
+        src.tiles = (const BatchTile*)bptr(b, b->B.tiles_off);
         src.base = b->mem;
         src.es = (int)elem_size(b->storage);
         src.cur = parity;
@@ -266,7 +266,7 @@ cudaError_t launch_batch_step(tvlbm_batch* b, int parity, cudaStream_t s) {
     BatchSrc src;
     src.dom = (const BatchDomain*)bptr(b, b->B.tables_off);
     src.maps = (const CUtensorMap*)bptr(b, b->B.maps_off);
-    src.tile_dom = (const int*)bptr(b, b->B.tiles_off);
+    src.tiles = (const BatchTile*)bptr(b, b->B.tiles_off);
     src.base = b->mem;
     src.ntiles = b->ntiles;
     src.parity = parity;

@@ -325,20 +325,29 @@ struct BatchDomain {
     float omegaf;
     double omegad;
 };
+// One tile of the batch's list: its origin and domain.  All that its window loads need is this record
+// (the domain's geometry is read while they are in flight); a domain index alone, with the origin
+// divided out of the domain's entry, put two more dependent reads ahead of them.
+struct BatchTile {
+    int x0, y0, dom, pad;
+};
+__device__ __forceinline__ BatchTile ld_tile(const BatchTile* t) {
+    const int4 v = __ldg(reinterpret_cast<const int4*>(t));
+    return {v.x, v.y, v.z, v.w};
+}
 struct BatchSrc {
     const BatchDomain* dom;
     const CUtensorMap* maps;  // [domain][buffer]
-    const int* tile_dom;
+    const BatchTile* tiles;
     unsigned char* base;
     int ntiles, parity, es;
     __device__ __forceinline__ void tile(int t, const KParams& p, int tx, int ty, int& x0, int& y0,
                                          const CUtensorMap*& map, void*& out, Geom& g) const {
-        const int d = __ldg(tile_dom + t);
-        const BatchDomain& D = dom[d];
-        const int local = t - D.tile_begin;
-        x0 = (local % D.tiles_x) * tx;
-        y0 = (local / D.tiles_x) * ty;
-        map = maps + 2 * d + parity;
+        const BatchTile r = ld_tile(tiles + t);
+        x0 = r.x0;
+        y0 = r.y0;
+        map = maps + 2 * r.dom + parity;
+        const BatchDomain& D = dom[r.dom];
         out = base + D.off[parity ^ 1] * es;
         g.nx = D.nx;
         g.ny = D.ny;
@@ -653,7 +662,7 @@ struct BatchFlowSrc {
     const BatchDomain* dom;
     const CUtensorMap* lmaps;  // [domain][buffer], window boxes
     const CUtensorMap* smaps;  // [domain][buffer], tile boxes
-    const int* tile_dom;
+    const BatchTile* tiles;
     unsigned char* base;
     int es, cur;               // element size; the buffer holding every domain's state at launch
     int ntiles, nsteps;
@@ -666,19 +675,19 @@ struct BatchFlowSrc {
 __device__ __forceinline__ void flow_task(const BatchFlowSrc& src, int task, int d, int& k, int& t, const int*& nb) {
     k = task / src.ntiles;
     t = task - k * src.ntiles;
-    const BatchDomain& D = src.dom[__ldg(src.tile_dom + t)];
+    const BatchDomain& D = src.dom[__ldg(&src.tiles[t].dom)];
     const int local = t - D.tile_begin;
     const int ty = local / D.tiles_x, tx = local - ty * D.tiles_x;
     nb = src.done + D.tile_begin + flow_neighbour(tx, ty, d, D.tiles_x, D.tiles_y);
 }
-__device__ __forceinline__ void flow_tile(const BatchFlowSrc& src, int t, int k, const KParams& p, int TX, int TY,
-                                          int& x0, int& y0, Geom& g, const CUtensorMap*& lmap,
-                                          const CUtensorMap*& smap, void*& out) {
-    const int d = __ldg(src.tile_dom + t);
+__device__ __forceinline__ void flow_tile(const BatchFlowSrc& src, int t, int k, const KParams& p, int, int, int& x0,
+                                          int& y0, Geom& g, const CUtensorMap*& lmap, const CUtensorMap*& smap,
+                                          void*& out) {
+    const BatchTile r = ld_tile(src.tiles + t);
+    const int d = r.dom;
     const BatchDomain& D = src.dom[d];
-    const int local = t - D.tile_begin;
-    x0 = (local % D.tiles_x) * TX;
-    y0 = (local / D.tiles_x) * TY;
+    x0 = r.x0;
+    y0 = r.y0;
     g.nx = D.nx;
     g.ny = D.ny;
     g.pitch = D.pitch;
