@@ -382,7 +382,7 @@ __device__ __forceinline__ void fv_march(const KParams& p, const FvParams& fp, i
     }
     if (fp.walls && y1 == p.ny) {
 #pragma unroll
-        for (int q = 0; q < PN; ++q) pend[q] = add2(src.own(q, p.ny - 1), pend[q]);
+        for (int q = 0; q < PN; ++q) pend[q] = add2(src.cur(q), pend[q]);
         put(p.ny - 1, pend);
     }
 }
@@ -481,16 +481,20 @@ __global__ void __launch_bounds__(32) fv_update_kernel(const typename C::T* __re
 // One kernel per step: a warp owns a strip of 30 output columns (lanes 0 and 31 hold the columns
 // beside it) and marches over a segment of rows: it loads a row's populations, computes the
 // collision term of its 32 cells in registers, takes the east and west neighbours' values by warp
-// shuffles and carries the row's contributions to the next rows (fv_march).  Nothing goes through
-// shared memory and the collision term never leaves the registers: Q values read and Q written per
-// cell update, 4 shuffles per velocity and cell where a block with both fields in shared memory
-// read 18 values, 1.07 x (seg + 2) / seg collision terms per output cell.  D2Q16 at 1024 x 1024 with
-// the Prandtl term: 57 us per step (91 us with a 32 x 16 block of both fields in shared memory, 1 873
-// instructions per cell, 35 us of it on the FP64 pipe converting double parameters); bound by the
-// FP32 pipe and the latency of 12 warps per SM (58 % of the issue slots).
+// shuffles and carries the row's contributions to the next rows (fv_march).  The collision term
+// never leaves the registers: Q values read and Q written per cell update, 4 shuffles per velocity
+// and cell where a block with both fields in shared memory read 18 values, 1.07 x (seg + 2) / seg
+// collision terms per output cell.  D2Q16 at 1024 x 1024 with the Prandtl term: 50 us per step (91 us
+// with a 32 x 16 block of both fields in shared memory, 1 873 instructions per cell, 35 us of it on
+// the FP64 pipe converting double parameters); bound by the FP32 pipe and issue, 20 us of memory
+// traffic underneath.
 template <int N1, class C>
-constexpr int fv_fused_minb() {  // resident CTAs of 128 threads (D2Q16: 168 registers; 4 CTAs at 128 spill and are slower)
-    return N1 == 3 ? 5 : N1 == 4 ? 3 : 2;
+constexpr int fv_fused_minb() {  // resident CTAs: 16 warps per SM (D2Q36: 8, 250 registers); a fifth
+    return 4;                     // for D2Q9 spills at 96 registers (41 against 39 us)
+}
+template <int N1>
+constexpr int fv_fused_warps() {  // warps per CTA; two for D2Q36, whose rings are 14 KB each
+    return N1 == 6 ? 2 : 4;
 }
 __device__ __forceinline__ Pair<float> shfl_e(Pair<float> v) {
     return {__shfl_down_sync(0xffffffffu, v.x, 1), __shfl_down_sync(0xffffffffu, v.y, 1)};
@@ -499,24 +503,60 @@ __device__ __forceinline__ Pair<float> shfl_w(Pair<float> v) {
     return {__shfl_up_sync(0xffffffffu, v.x, 1), __shfl_up_sync(0xffffffffu, v.y, 1)};
 }
 
-// Row source of the fused form: the lane's cell in registers, its neighbours by shuffles.
+// Row source of the fused form: the lane's cell in registers, its neighbours by shuffles.  Rows come
+// through a ring of three slots in shared memory that each lane fills for itself (asynchronous copies,
+// no barrier: a lane reads only what it copied): the next row is in flight while this one is computed,
+// which registers had no room for, and the row before it is still there when its output is completed,
+// so its f_0 needs no registers either and D2Q16 fits four CTAs.  Against loads into registers at the
+// head of each row, us per step at 1024 x 1024: D2Q9 44 -> 39, D2Q16 57.5 -> 50, D2Q36 134 -> 112; 64 x 61:
+// 6.6 -> 6.0, 6.3 -> 6.4, 9.0 -> 10.1.
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
 template <int N1, class C>
 struct FvStripSrc {
     using R = typename C::R;
-    static constexpr bool kCarry = N1 <= 4;  // D2Q36: 36 more registers would spill, f_0 is read again
+    static constexpr bool kCarry = false;
+    static constexpr int SLOT = N1 * N1 * 32;  // elements of a warp's row
     const typename C::T* f;  // the column's element of row 0 in plane 0
     const KParams& p;
     const FvParams& fp;
+    R* ring;  // [3][Q][32], at this lane
+    int next, last, slot;  // the row whose copy is started next, the last one; the current row's slot
     Pair<R> s[fv_hp<N1>()][N1], o[fv_hp<N1>()][N1];
-    __device__ __forceinline__ Pair<R> cur(int q) const { return s[q / N1][q % N1]; }
-    __device__ __forceinline__ Pair<R> own(int q, int y) const {  // still in the L1 cache
-        const typename C::T* b = f + (long long)y * p.pitch;
-        const int i = q % N1, g = q / N1;
-        return {(R)C::ld(b + (long long)(i + N1 * g) * p.plane),
-                fv_single<N1>(g) ? R(0) : (R)C::ld(b + (long long)(i + N1 * (N1 - 1 - g)) * p.plane)};
+    __device__ __forceinline__ void start(int sl) {
+        if (next <= last) {
+            const typename C::T* b = f + (long long)next * p.pitch;
+#pragma unroll
+            for (int l = 0; l < N1 * N1; ++l) {
+                cp_async4(ring + sl * SLOT + l * 32, b);
+                b += p.plane;
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        ++next;
     }
-    __device__ __forceinline__ void row(int r) {
-        fv_load_cell<N1, C>(f + (long long)r * p.pitch, p.plane, s);
+    __device__ __forceinline__ void begin(int first, int last_) {
+        next = first;
+        last = last_;
+        slot = 2;
+        start(0);
+    }
+    __device__ __forceinline__ Pair<R> at(const R* b, int q) const {
+        const int i = q % N1, g = q / N1;
+        return {b[(i + N1 * g) * 32], fv_single<N1>(g) ? R(0) : b[(i + N1 * (N1 - 1 - g)) * 32]};
+    }
+    __device__ __forceinline__ Pair<R> cur(int q) const { return s[q / N1][q % N1]; }
+    __device__ __forceinline__ Pair<R> own(int q, int) const { return at(ring + (slot == 0 ? 2 : slot - 1) * SLOT, q); }
+    __device__ __forceinline__ void row(int) {
+        slot = slot == 2 ? 0 : slot + 1;
+        start(slot == 2 ? 0 : slot + 1);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        const R* b = ring + slot * SLOT;
+#pragma unroll
+        for (int g = 0; g < fv_hp<N1>(); ++g)
+#pragma unroll
+            for (int i = 0; i < N1; ++i) s[g][i] = at(b, g * N1 + i);
         fv_omega_cell<N1, R>(s, p, fp, o);
     }
     __device__ __forceinline__ void get(int q, Pair<R>& f0, Pair<R>& fE, Pair<R>& fW, Pair<R>& o0, Pair<R>& oE,
@@ -531,14 +571,14 @@ struct FvStripSrc {
 };
 
 template <int N1, class C>
-__global__ void __launch_bounds__(128, fv_fused_minb<N1, C>())
+__global__ void __launch_bounds__(fv_fused_warps<N1>() * 32, fv_fused_minb<N1, C>())
     fv_fused_kernel(const typename C::T* __restrict__ f, typename C::T* __restrict__ fout, const KParams p,
                     const FvParams fp, int strips, int seg) {
     using R = typename C::R;
     constexpr int HP = fv_hp<N1>(), PN = HP * N1;
     pdl_launch_dependents();
     pdl_wait();
-    const int w = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int w = blockIdx.x * fv_fused_warps<N1>() + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     const int strip = w % strips, y0 = (w / strips) * seg;
     if (y0 >= p.ny) return;  // whole warps
     const int y1 = min(y0 + seg, p.ny);
@@ -546,7 +586,9 @@ __global__ void __launch_bounds__(128, fv_fused_minb<N1, C>())
     const int xl = min(x, p.nx);  // columns beyond the frame column nx belong to no output
     const bool mine = lane >= 1 && lane <= 30 && x < p.nx;
     const Geom geo = geom_of(p);
-    FvStripSrc<N1, C> src{f + sidx(p, 0, xl, 0), p, fp};
+    __shared__ R ring[fv_fused_warps<N1>()][3 * FvStripSrc<N1, C>::SLOT];
+    FvStripSrc<N1, C> src{f + sidx(p, 0, xl, 0), p, fp, &ring[threadIdx.x >> 5][lane]};
+    src.begin(fp.walls ? max(y0 - 1, 0) : y0 - 1, fp.walls ? min(y1, p.ny - 1) : y1);
     const auto put = [&](int y, const Pair<R>(&out)[PN]) {
         if (!mine) return;
         R s[N1 * N1];
@@ -885,7 +927,8 @@ cudaError_t launch_fv(const void* f, void* om, void* fout, const KParams& p, con
         return launch_as(false, fv_update64_kernel<N1>, dim3((unsigned)(gx * p.ny), N1 * N1), dim3(32), 0, s, (const T*)f,
                           (const T*)om, (T*)fout, p, fp);
     } else {
-        const long long warps = 4LL * fv_fused_minb<N1, C>() * sms;  // resident warps of the fused form
+        constexpr int W = fv_fused_warps<N1>();
+        const long long warps = (long long)W * fv_fused_minb<N1, C>() * sms;  // resident warps of the fused form
         if (fp.walls) e = launch_pdl(fv_impose_kernel<N1, C>, dim3((2 * p.nx + 31) / 32), dim3(32), 0, s, (T*)f, p, wp);
         if (e != cudaSuccess) return e;
         if (split) {
@@ -901,8 +944,8 @@ cudaError_t launch_fv(const void* f, void* om, void* fout, const KParams& p, con
         long long seg = ((long long)strips * p.ny + warps - 1) / warps;
         seg = seg < 1 ? 1 : (seg > 32 ? 32 : seg);
         const long long n = strips * ((p.ny + seg - 1) / seg);
-        return launch_pdl(fv_fused_kernel<N1, C>, dim3((unsigned)((n + 3) / 4)), dim3(128), 0, s, (const T*)f, (T*)fout, p,
-                          fp, strips, (int)seg);
+        return launch_pdl(fv_fused_kernel<N1, C>, dim3((unsigned)((n + W - 1) / W)), dim3(W * 32), 0, s, (const T*)f,
+                          (T*)fout, p, fp, strips, (int)seg);
     }
 }
 
