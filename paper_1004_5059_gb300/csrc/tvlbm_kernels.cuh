@@ -254,6 +254,13 @@ __device__ __forceinline__ typename C::R split_rest(const KParams& p, int l, typ
     if constexpr (C::split) return v - p.Whi[l]; else return v;
 }
 
+// The stored value at byte offset off of a plane (32-bit offsets from a uniform base: one instruction
+// per load where 64-bit addresses take three; a plane of 4 GB or more takes 64-bit ones).
+template <class C, class Off>
+__device__ __forceinline__ typename C::R ld_at(const typename C::T* base, Off off) {
+    return C::ld(reinterpret_cast<const typename C::T*>(reinterpret_cast<const char*>(base) + off));
+}
+
 // Storage value -> f_l and back, in precision R (used off the hot path: init, moments,
 // reductions, walls); ref = R_l, the deviation reference of velocity l.
 template <class C, class R>

@@ -45,22 +45,16 @@ __device__ __forceinline__ const R* wall_lengths(const MeshDev& m) {
 // shuffle instead of two loads per source row.  KT > 0: every row's list padded to KT entries (padding: weight
 // 0 on the row's first source), unrolled so that all loads of a velocity are in flight together;
 // KT = 0: a loop that ends at the first zero weight.  Both add the same terms in the same order.
-// 1024 x 1024 D2Q16 FP32 deviations on the tanh channel (lists of 3): 41 us per step, wall fill included;
-// 56 us with two loads per source row, 64-bit addresses and launches that do not overlap.
+// 1024 x 1024 D2Q16 FP32 deviations on the tanh channel (lists of 3): 40 us per step, wall fill included
+// (43 us with 256-thread CTAs, which fit 24 warps where 128-thread ones fit 28; 56 us with two loads per
+// source row, 64-bit addresses and launches that do not overlap).
 template <int N1, class C>
-constexpr int mesh_sweep_minb() {  // resident CTAs of 256 threads: 3 (85 registers) for FP32 up to D2Q16
-    return (sizeof(typename C::R) == 4 && N1 <= 4) ? 3 : 1;
+constexpr int mesh_sweep_minb() {  // resident CTAs of 128 threads: 7 (72 registers, 28 warps) for FP32 up to D2Q16
+    return (sizeof(typename C::R) == 4 && N1 <= 4) ? 7 : 1;
 }
 
-// The stored value at byte offset off of a plane (32-bit offsets from a uniform base: one instruction
-// per load where 64-bit addresses take three; a plane of 4 GB or more takes 64-bit ones).
-template <class C, class Off>
-__device__ __forceinline__ typename C::R ld_at(const typename C::T* base, Off off) {
-    return C::ld(reinterpret_cast<const typename C::T*>(reinterpret_cast<const char*>(base) + off));
-}
-
-template <int N1, class C, int KT, class Off = unsigned>
-__global__ void __launch_bounds__(256, mesh_sweep_minb<N1, C>()) mesh_sweep_kernel(const typename C::T* __restrict__ fin,
+template <int N1, class C, int KT, class Off = unsigned, int BR = 4>
+__global__ void __launch_bounds__(32 * BR, BR == 4 ? mesh_sweep_minb<N1, C>() : 1) mesh_sweep_kernel(const typename C::T* __restrict__ fin,
                                                          typename C::T* __restrict__ fout, const KParams p,
                                                          const MeshDev m) {
     using R = typename C::R;
@@ -223,10 +217,10 @@ cudaError_t step_as(const void* fin, void* fout, const KParams& p, const MeshDev
         const cudaError_t e = launch_pdl(mesh_wall_kernel<N1, C>, grid, block, 0, s, (T*)fin, p, m);
         if (e != cudaSuccess) return e;
     }
-    const dim3 block(32, 8), grid((p.nx + 30) / 31, (p.ny + 7) / 8);
     // the table's row length m.k is the longest list; shorter lists are padded to it
-    const bool wide = (unsigned long long)p.plane * sizeof(T) >> 32 != 0;
-    const auto kernel = wide       ? mesh_sweep_kernel<N1, C, 0, unsigned long long>
+    const bool wide = (unsigned long long)p.plane * sizeof(T) >> 32 != 0 || p.ny > 4 * 65535;  // (the grid's y extent)
+    const dim3 block(32, wide ? 8 : 4), grid((p.nx + 30) / 31, (p.ny + block.y - 1) / block.y);
+    const auto kernel = wide       ? mesh_sweep_kernel<N1, C, 0, unsigned long long, 8>
                         : m.k <= 2 ? mesh_sweep_kernel<N1, C, 2>
                         : m.k == 3 ? mesh_sweep_kernel<N1, C, 3>
                         : m.k == 4 ? mesh_sweep_kernel<N1, C, 4>
