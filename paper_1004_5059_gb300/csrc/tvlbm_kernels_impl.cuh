@@ -19,32 +19,68 @@ namespace tvlbm {
 // and wall ghost rows live in the stored frame, so no index wraps here.
 // =============================================================================================
 // ROWS: the launch has a per-row deviation reference (chosen at launch, as for the tiled form).
-template <int N1, class C, bool ROWS>
-__global__ void __launch_bounds__(256) sweep_plain_kernel(const typename C::T* __restrict__ fin,
-                                                          typename C::T* __restrict__ fout, const KParams p) {
+// SHUFFLE (FP32 arithmetic, D2Q16 and D2Q36): a warp takes 31 columns of a row, its lane 0 the source
+// column left of them; the values one column to the left come from the neighbouring lane, so a
+// velocity costs two loads with 32-bit offsets and two shuffles instead of four loads: the same
+// arithmetic on the same values.
+template <int N1, bool SHUFFLE>
+constexpr int sweep_plain_minb() {  // resident CTAs of 128 threads: 7 for D2Q16 (72 registers), 4 for D2Q36
+    return !SHUFFLE ? 1 : N1 == 4 ? 7 : 4;
+}
+template <int N1, class C, bool ROWS, bool SHUFFLE>
+__global__ void __launch_bounds__(SHUFFLE ? 128 : 256, sweep_plain_minb<N1, SHUFFLE>())
+    sweep_plain_kernel(const typename C::T* __restrict__ fin, typename C::T* __restrict__ fout, const KParams p) {
     using R = typename C::R;
     using T = typename C::T;
-    constexpr int Q = N1 * N1;
+    constexpr int Q = N1 * N1, H = N1 / 2;
+    static_assert(!SHUFFLE || (sizeof(R) == 4 && N1 % 2 == 0));
     pdl_launch_dependents();
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int x = SHUFFLE ? (int)(blockIdx.x * 31 + threadIdx.x) - 1 : (int)(blockIdx.x * 32 + threadIdx.x);
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     pdl_wait();  // the previous step's populations are complete from here on
-    if (x >= p.nx || y >= p.ny) return;
+    if (y >= p.ny || (!SHUFFLE && x >= p.nx)) return;  // (whole warps where lanes exchange values)
     R s[Q];
+    if constexpr (SHUFFLE) {
+        using Off = unsigned;
+        const Off xo = (Off)(min(x, p.nx - 1) + p.hx);
 #pragma unroll
-    for (int j = 0; j < N1; ++j) {
-        const R ay = ka<R>(p, j);
-        const int ys = y + HY - p.sh[j];
+        for (int j = 0; j < N1; ++j) {
+            const R ay = ka<R>(p, j);
+            // byte offsets of the two source rows in a plane
+            const Off o0 = ((Off)(y + HY - p.sh[j]) * (Off)p.pitch + xo) * (Off)sizeof(T), o1 = o0 - (Off)p.pitch * (Off)sizeof(T);
 #pragma unroll
-        for (int i = 0; i < N1; ++i) {
-            const R ax = ka<R>(p, i);
-            const int xs = x + p.hx - p.sh[i];
-            const T* b = fin + (long long)(i + N1 * j) * p.plane + (long long)ys * p.pitch + xs;
-            const R v00 = C::ld(b), v01 = C::ld(b - 1);
-            const R v10 = C::ld(b - p.pitch), v11 = C::ld(b - p.pitch - 1);
-            const R r0 = fma(ax, v01 - v00, split_rest<C>(p, i + N1 * j, v00));
-            const R r1 = fma(ax, v11 - v10, split_rest<C>(p, i + N1 * j, v10));
-            s[i + N1 * j] = fma(ay, r1 - r0, r0);
+            for (int i = 0; i < H; ++i) {  // the mirror pair (i, N1 - 1 - i) in packed arithmetic
+                const int mi = N1 - 1 - i, l = i + N1 * j, lm = mi + N1 * j;
+                const T *ca = fin + ((long long)l * p.plane - p.sh[i]), *cb = fin + ((long long)lm * p.plane - p.sh[mi]);
+                const float2 v0 = make_float2(ld_at<C, Off>(ca, o0), ld_at<C, Off>(cb, o0));
+                const float2 v1 = make_float2(ld_at<C, Off>(ca, o1), ld_at<C, Off>(cb, o1));
+                const float2 w0 = make_float2(__shfl_up_sync(0xffffffffu, v0.x, 1), __shfl_up_sync(0xffffffffu, v0.y, 1));
+                const float2 w1 = make_float2(__shfl_up_sync(0xffffffffu, v1.x, 1), __shfl_up_sync(0xffffffffu, v1.y, 1));
+                const float2 ax = make_float2(ka<R>(p, i), ka<R>(p, mi));
+                const float2 r0 = __ffma2_rn(ax, f2sub(w0, v0), make_float2(split_rest<C>(p, l, v0.x), split_rest<C>(p, lm, v0.y)));
+                const float2 r1 = __ffma2_rn(ax, f2sub(w1, v1), make_float2(split_rest<C>(p, l, v1.x), split_rest<C>(p, lm, v1.y)));
+                const float2 o = __ffma2_rn(make_float2(ay, ay), f2sub(r1, r0), r0);
+                s[l] = o.x;
+                s[lm] = o.y;
+            }
+        }
+        if (threadIdx.x == 0 || x >= p.nx) return;
+    } else {
+#pragma unroll
+        for (int j = 0; j < N1; ++j) {
+            const R ay = ka<R>(p, j);
+            const int ys = y + HY - p.sh[j];
+#pragma unroll
+            for (int i = 0; i < N1; ++i) {
+                const R ax = ka<R>(p, i);
+                const int xs = x + p.hx - p.sh[i];
+                const T* b = fin + (long long)(i + N1 * j) * p.plane + (long long)ys * p.pitch + xs;
+                const R v00 = C::ld(b), v01 = C::ld(b - 1);
+                const R v10 = C::ld(b - p.pitch), v11 = C::ld(b - p.pitch - 1);
+                const R r0 = fma(ax, v01 - v00, split_rest<C>(p, i + N1 * j, v00));
+                const R r1 = fma(ax, v11 - v10, split_rest<C>(p, i + N1 * j, v10));
+                s[i + N1 * j] = fma(ay, r1 - r0, r0);
+            }
         }
     }
     const Geom g = geom_of(p);
@@ -107,11 +143,14 @@ __global__ void __launch_bounds__(32) sweep_lanes_kernel(const double* __restric
 // The tiled form runs small domains without tiles (the same bits).  A tile's windows take a TMA round
 // trip and its threads walk 2 to 4 rows one after another, which a small grid has no other work to
 // hide: 100 x 75 D2Q9 FP32 4.9 us per step tiled against 2.5 with one cell per thread, 128 x 128
-// D2Q16 6.4 against 2.9.  The line lies where the tiles' fewer loads (each value once, not four times
-// through the L1 cache) begin to pay: at 12 M populations in 4-byte storage (768 x 768 D2Q16 15.3
-// against 16.8 us, 1000 x 601 17.5 against 19.0; 1024 x 1024 30.8 against 30.7) and 8 M in 2-byte
-// storage, whose single loads carry half as much (600 x 600 D2Q16 11.0 against 11.6 us; 1024 x 512
-// D2Q36 40 against 35.5).  FP64 is bound by its arithmetic, so what counts is an even spread over the
+// D2Q16 6.4 against 2.9.  The line lies where the tiles' fewer loads (each value once, not twice or four
+// times through the L1 cache) and whole-row stores begin to pay: at 15 M populations in 4-byte storage
+// (without tiles against tiled: 1000 x 601 D2Q16 FP32 15.3 against 19.0 us, 960 x 960 27.4 against 27.7,
+// 1024 x 1024 34 against 31; 640 x 600 D2Q36 29.5 against 33.6), in 2-byte storage, whose single loads carry
+// half as much, at 8 M for D2Q9 (1000 x 950 15.2 against 16.0, 1300 x 1300 25.0 against 23.6), 15 M for
+// D2Q16 (768 x 768 14.7 against 16.7, 980 x 980 22.5 against 22.7) and 30 M for D2Q36, where the tiles'
+// windows leave few warps (channels: 1024 x 512 33.6 against 38.3, 1000 x 900 57.1 against 58.7, 2048 x 512
+// 63.2 against 62.2).  FP64 is bound by its arithmetic, so what counts is an even spread over the
 // SM partitions: blocks of one warp, launched without programmatic overlap (blocks placed around those
 // of a kernel still resident share partitions: 64 x 64 D2Q16 8.5 instead of 5.6 us, 256 x 256 59
 // instead of 37), up to 600 cells per SM (256 x 256 37 against 51 to 72 us tiled; 500 x 300 79.7 against
@@ -130,7 +169,19 @@ inline bool sweep_without_tiles(const KParams& p) {
     const long long cells = (long long)p.nx * p.ny;
     if (p.ny > 65535) return false;  // rows of blocks: the grid's y extent
     if (sizeof(typename C::T) == 8) return cells <= 600LL * sm_count();
-    return cells * (N1 * N1) <= (sizeof(typename C::T) == 4 ? 12000000LL : 8000000LL);
+    return cells * (N1 * N1) <= (sizeof(typename C::T) == 4 || N1 == 4 ? 15000000LL : N1 == 3 ? 8000000LL : 30000000LL);
+}
+// The shuffled gather where the cells are more than the resident warps' (below, the extra latency
+// counts: D2Q16 FP32 360 x 300 5.0 against 4.4 us with four loads, 512 x 512 7.9 against 8.2; D2Q36 FP32 200 x 150
+// 5.8 against 5.2, 256 x 256 6.3 against 7.0) and both buffers stay in the L2 cache (1000 x 601 D2Q16 FP32
+// 15.3 against 16.9, 768 x 768 FP16 14.7 against 16.0, D2Q36 512 x 512 FP32 16.8 against 19.1, 400 x 500 FP16
+// 12.6 against 15.8): beyond it the 31-column rows, whose stores share sectors between blocks, cost
+// memory traffic (1024 x 1024 FP32 32.7 against 30.8).  D2Q9 has too little to load (1000 x 601 10.3
+// either way).
+template <int N1, class C>
+inline bool sweep_by_shuffle(const KParams& p) {
+    const long long cells = (long long)p.nx * p.ny;
+    return cells >= (N1 == 4 ? 250000 : 64000) && 2 * cells * (N1 * N1) * (long long)sizeof(typename C::T) <= 125000000LL;
 }
 template <int N1>
 inline bool sweep_in_lanes(const KParams& p) {
@@ -587,10 +638,22 @@ struct Launch {
         // blocks of 128 threads: 3 to 8 % faster than 256 from 128 x 128 to 1024 x 1024 (D2Q36 channels
         // up to 30 %); one warp in FP64 (see above)
         const dim3 b(32, p.ny > 4 * 65535 ? 8 : (F64 && p.ny <= 65535) ? 1 : 4);
-        if constexpr (C::dev) {
-            if (p.rowf) return launch_pdl(sweep_plain_kernel<N1, C, true>, grid2d(p, b), b, 0, s, (const T*)fin, (T*)fout, p);
+        const auto launch = [&](auto kernel, int cols) {
+            const dim3 grid((p.nx + cols - 1) / cols, (p.ny + b.y - 1) / b.y);
+            return launch_as(!F64, kernel, grid, b, 0, s, (const T*)fin, (T*)fout, p);
+        };
+        if constexpr (!F64 && N1 >= 4) {
+            if (b.y == 4 && sweep_by_shuffle<N1, C>(p)) {
+                if constexpr (C::dev) {
+                    if (p.rowf) return launch(sweep_plain_kernel<N1, C, true, true>, 31);
+                }
+                return launch(sweep_plain_kernel<N1, C, false, true>, 31);
+            }
         }
-        return launch_as(!F64, sweep_plain_kernel<N1, C, false>, grid2d(p, b), b, 0, s, (const T*)fin, (T*)fout, p);
+        if constexpr (C::dev) {
+            if (p.rowf) return launch(sweep_plain_kernel<N1, C, true, false>, 32);
+        }
+        return launch(sweep_plain_kernel<N1, C, false, false>, 32);
     }
     template <class C>
     static cudaError_t init_c(const double* fields, void* f, const KParams& p, cudaStream_t s) {
