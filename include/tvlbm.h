@@ -66,7 +66,8 @@ extern "C" {
 /* ---- sweep kernel forms ------------------------------------------------------------------ */
 #define TVLBM_FORM_PLAIN 0 /* one thread per cell, direct gathers from global memory           */
 #define TVLBM_FORM_TILED 1 /* 2-D tiles whose per-velocity source windows are staged in shared
-                              memory by TMA; the default                                       */
+                              memory by TMA; the default (small domains run without tiles: the
+                              same populations)                                                */
 #define TVLBM_FORM_FLOW 2  /* the tiled sweep of several time steps in one persistent launch: a
                               tile starts a step as soon as its 3 x 3 periodic neighbourhood has
                               finished the previous one (no launch boundary between steps).
