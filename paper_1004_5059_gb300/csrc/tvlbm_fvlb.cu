@@ -428,26 +428,42 @@ __global__ void __launch_bounds__(32) fv_omega_kernel(const typename C::T* __res
     store_collided<N1, C>(om, geom_of(p), x, y, o);
 }
 
-// Row source of the update: a pair of velocities of both fields in memory.
+// Row source of the update: a pair of velocities of both fields in memory (two: false for a y-node
+// without a mirror, whose second lane of the pair is not used).
 template <class C>
 struct FvGlobalSrc {
     using R = typename C::R;
     static constexpr bool kCarry = true;
     const typename C::T *fa, *fb, *oa, *ob;  // the column's elements of row 0
     long long pitch, at;
-    __device__ __forceinline__ void row(int r) { at = r * pitch; }
-    __device__ __forceinline__ Pair<R> cur(int) const { return {(R)C::ld(fa + at), (R)C::ld(fb + at)}; }
-    __device__ __forceinline__ Pair<R> own(int, int y) const {
-        return {(R)C::ld(fa + y * pitch), (R)C::ld(fb + y * pitch)};
+    bool two;
+    Pair<R> f0, fE, fW, o0, oE, oW;
+    __device__ __forceinline__ void row(int r) {
+        at = r * pitch;
+        f0.x = C::ld(fa + at);
+        fE.x = C::ld(fa + at + 1);
+        fW.x = C::ld(fa + at - 1);
+        o0.x = C::ld(oa + at);
+        oE.x = C::ld(oa + at + 1);
+        oW.x = C::ld(oa + at - 1);
+        if (two) {
+            f0.y = C::ld(fb + at);
+            fE.y = C::ld(fb + at + 1);
+            fW.y = C::ld(fb + at - 1);
+            o0.y = C::ld(ob + at);
+            oE.y = C::ld(ob + at + 1);
+            oW.y = C::ld(ob + at - 1);
+        }
     }
-    __device__ __forceinline__ void get(int, Pair<R>& f0, Pair<R>& fE, Pair<R>& fW, Pair<R>& o0, Pair<R>& oE,
-                                        Pair<R>& oW) const {
-        f0 = {(R)C::ld(fa + at), (R)C::ld(fb + at)};
-        fE = {(R)C::ld(fa + at + 1), (R)C::ld(fb + at + 1)};
-        fW = {(R)C::ld(fa + at - 1), (R)C::ld(fb + at - 1)};
-        o0 = {(R)C::ld(oa + at), (R)C::ld(ob + at)};
-        oE = {(R)C::ld(oa + at + 1), (R)C::ld(ob + at + 1)};
-        oW = {(R)C::ld(oa + at - 1), (R)C::ld(ob + at - 1)};
+    __device__ __forceinline__ Pair<R> cur(int) const { return f0; }
+    __device__ __forceinline__ Pair<R> own(int, int) const { return f0; }  // (carried by the march)
+    __device__ __forceinline__ void get(int, Pair<R>& f, Pair<R>& e, Pair<R>& w, Pair<R>& o, Pair<R>& p, Pair<R>& q) const {
+        f = f0;
+        e = fE;
+        w = fW;
+        o = o0;
+        p = oE;
+        q = oW;
     }
 };
 
@@ -469,7 +485,8 @@ __global__ void __launch_bounds__(32) fv_update_kernel(const typename C::T* __re
     const int la = i + N1 * g, lb = single ? la : i + N1 * (N1 - 1 - g);
     const Geom geo = geom_of(p);
     FvGlobalSrc<C> src{f + sidx(p, la, x, 0), f + sidx(p, lb, x, 0), om + sidx(p, la, x, 0), om + sidx(p, lb, x, 0),
-                       (long long)p.pitch, 0};
+                       (long long)p.pitch, 0, !single};
+    src.f0 = src.fE = src.fW = src.o0 = src.oE = src.oW = Pair<R>{R(0), R(0)};
     const auto put = [&](int y, const Pair<R>(&out)[1]) {
         store_with_images(fout, geo, (long long)la * p.plane, x, y, C::enc(out[0].x));
         if (!single) store_with_images(fout, geo, (long long)lb * p.plane, x, y, C::enc(out[0].y));
@@ -934,7 +951,12 @@ cudaError_t launch_fv(const void* f, void* om, void* fout, const KParams& p, con
         if (split) {
             e = launch_pdl(fv_omega_kernel<N1, C>, dim3((unsigned)(gx * p.ny)), dim3(32), 0, s, (const T*)f, (T*)om, p, fp);
             if (e != cudaSuccess) return e;
-            constexpr int seg = 8;  // rows per thread: the rows above and below a segment are taken again
+            // rows per thread: what fills 32 one-warp CTAs per SM, up to 8 (the rows above and below a
+            // segment are taken again; D2Q9 FP32 per step, 8 rows always against this: 64 x 61 13.3 and 6.5 us,
+            // 300 x 200 16.5 and 11.9)
+            const long long pairs = fv_hp<N1>() * N1;
+            int seg = (int)((gx * p.ny * pairs + 32LL * sms - 1) / (32LL * sms));
+            seg = seg < 1 ? 1 : (seg > 8 ? 8 : seg);
             return launch_pdl(fv_update_kernel<N1, C>, dim3((unsigned)(gx * ((p.ny + seg - 1) / seg)), fv_hp<N1>() * N1),
                               dim3(32), 0, s, (const T*)f, (const T*)om, (T*)fout, p, fp, seg);
         }
