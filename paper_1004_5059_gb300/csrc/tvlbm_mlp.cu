@@ -704,7 +704,10 @@ __global__ void __launch_bounds__(64) reduce_gradient_kernel(const float* __rest
         return;
     }
     // a bias per warp, its lanes sharing the CTAs' row groups, in compensated FP32 (each addition's
-    // rounding error is kept by the two-sum identity; FP64 would take 64 cycles a warp instruction)
+    // rounding error is kept by the two-sum identity; FP64 would take 64 cycles a warp instruction).
+    // The last bit of a bias flips a BF16 rounding now and then, and a training run amplifies that (4096
+    // rows, 16 iterations: gradients up to 3e-4 apart, as two runs with atomic sums were); plain sums
+    // in row order lie further from either.
     const int k = (t - Cfg::P_SUM) >> 5, lane = threadIdx.x & 31;  // b1, b2, b3
     if (k >= 2 * NH + NOUT) return;
     const int boff = k < NH ? Cfg::P_B1 + k : k < 2 * NH ? Cfg::P_B2 + k - NH : Cfg::P_B3 + k - 2 * NH;
