@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(kFusedThreads, 3) mlp_fused_forward_kernel(con
                                                                 int* status, const MlpFeatures feat) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* base = smem_raw + ((1024u - (saddr(smem_raw) & 1023u)) & 1023u);
-    __shared__ uint64_t load_bar, mma_bar;
+    __shared__ uint64_t load_bar, mma_bar, end_bar;
     __shared__ uint32_t tmem_slot;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int m0 = blockIdx.x * BM;
@@ -216,6 +216,7 @@ __global__ void __launch_bounds__(kFusedThreads, 3) mlp_fused_forward_kernel(con
     if (tid == 0) {
         bar_init(&load_bar, 1);
         bar_init(&mma_bar, 1);
+        bar_init(&end_bar, 1);
         bar_init_fence();
     }
     if (warp == 0) tmem_alloc(&tmem_slot, FusedCfg::TMEM_COLS);
@@ -342,8 +343,12 @@ __global__ void __launch_bounds__(kFusedThreads, 3) mlp_fused_forward_kernel(con
             for (int e = 0; e < 4; ++e) o[e] = 4 * q + e < NOUT ? v[4 * q + e] + __ldcg(b3 + 4 * q + e) : 0.0f;
             d[q] = make_float4(o[0], o[1], o[2], o[3]);
         }
-    } else if (tid == 0 && status) {
-        atomicOr(status, 1);
+    } else if (tid == 0 && !ok) {
+        if (status) atomicOr(status, 1);
+        // let the loads and products started so far end before the CTA exits (bounded)
+        bar_wait(&load_bar, 0);
+        mma_commit(&end_bar);
+        bar_wait(&end_bar, 0);
     }
     tc_fence_before();
     __syncthreads();
@@ -415,7 +420,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) mlp_train_kernel(const __gri
     static_assert(kFusedGroups == 4, "32 columns per thread and hidden layer");
     extern __shared__ unsigned char smem_raw[];
     unsigned char* base = smem_raw + ((1024u - (saddr(smem_raw) & 1023u)) & 1023u);
-    __shared__ uint64_t w_bar, x_bar, mma_bar;
+    __shared__ uint64_t w_bar, x_bar, mma_bar, end_bar;
     __shared__ __align__(16) float bias[2 * NH + NOUTP];
     __shared__ uint32_t tmem_slot;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -424,6 +429,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) mlp_train_kernel(const __gri
         bar_init(&w_bar, 1);
         bar_init(&x_bar, 1);
         bar_init(&mma_bar, 1);
+        bar_init(&end_bar, 1);
         bar_init_fence();
     }
     pdl_wait();  // the weights (and the partial sums' readers) of the kernels before this one
@@ -456,7 +462,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) mlp_train_kernel(const __gri
         bar_expect_tx(&x_bar, Cfg::TX_X);
         tma_load_2d(xs, &mx, &x_bar, 0, (int)blockIdx.x * BM);
     }
-    uint32_t ph = 0;  // phase of mma_bar
+    uint32_t ph = 0;   // phase of mma_bar
+    uint32_t xph = 0;  // phase of x_bar that the last input tile issued completes
     bool ok = true;
     // every thread waits for the products committed last; the MMAs' reads of shared memory are done too
     auto products_done = [&]() {
@@ -485,7 +492,6 @@ __global__ void __launch_bounds__(kFusedThreads, 1) mlp_train_kernel(const __gri
 #pragma unroll 1
     for (int tile = blockIdx.x; ok && tile < tiles; tile += gridDim.x, first = false) {
         const int m0 = tile * BM;
-        const uint32_t xph = (uint32_t)((tile - (int)blockIdx.x) / (int)gridDim.x) & 1u;
         float4 ys[3];
         if (warp < 4) {  // the targets, long before they are needed
             const float* q = ystar + (size_t)(m0 + r) * NOUTP;
@@ -627,6 +633,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) mlp_train_kernel(const __gri
         if (tid == 0 && ok && tile + (int)gridDim.x < tiles) {
             bar_expect_tx(&x_bar, Cfg::TX_X);
             tma_load_2d(xs, &mx, &x_bar, 0, (tile + (int)gridDim.x) * BM);
+            xph ^= 1;
         }
     }
 
@@ -656,9 +663,11 @@ __global__ void __launch_bounds__(kFusedThreads, 1) mlp_train_kernel(const __gri
         qb[Cfg::P_B2 + (warp & 3) * NH + cbeg + lane] = db2;
     } else if (tid == 0) {
         if (status) atomicOr(status, 1);
-        // let the loads started so far land before the CTA exits (bounded)
+        // let the loads and products started so far end before the CTA exits (bounded)
         bar_wait(&w_bar, 0);
-        bar_wait(&x_bar, 0);
+        bar_wait(&x_bar, xph);
+        mma_commit(&end_bar);
+        bar_wait(&end_bar, 0);
     }
     tc_fence_before();
     __syncthreads();

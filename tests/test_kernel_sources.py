@@ -1,0 +1,44 @@
+"""Rules of the kernels that no run can show, checked on their source text."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1004_5059_gb300", "csrc")
+
+
+def source(name):
+    text = open(os.path.join(CSRC, name)).read()
+    return re.sub(r"//[^\n]*", "", text)
+
+
+def body_of(text, name):
+    """The text between the braces of the function `name`."""
+    at = text.index("{", re.search(r"%s\s*\([^;]*?\)\s*\{" % name, text).end() - 1)
+    depth = 0
+    for k in range(at, len(text)):
+        depth += {"{": 1, "}": -1}.get(text[k], 0)
+        if depth == 0:
+            return text[at:k + 1]
+    raise AssertionError(name)
+
+
+def test_a_network_kernel_that_gives_up_waits_for_its_copies_and_products():
+    """A CTA must not exit with a bulk copy into its shared memory or a product in flight.  A barrier's
+    wait for parity q returns at once while the phase in progress has the other parity, so the wait for
+    the last of several loads on one barrier needs the parity of that load: it flips with every issue."""
+    text = source("tvlbm_mlp.cu")
+    train = body_of(text, "mlp_train_kernel")
+    first, later = [m.end() for m in re.finditer(r"tma_load_2d\(xs, &mx, &x_bar, [^;]*;", train)]
+    assert re.match(r"\s*xph \^= 1;", train[later:])
+    assert train.count("xph ^= 1") == 1 and re.search(r"uint32_t xph = 0;", train)
+    gave_up = train[train.index("atomicOr(status, 1)"):]
+    assert re.search(r"bar_wait\(&w_bar, 0\);\s*bar_wait\(&x_bar, xph\);\s*mma_commit\(&end_bar\);\s*bar_wait\(&end_bar, 0\);", gave_up)
+    forward = body_of(text, "mlp_fused_forward_kernel")
+    gave_up = forward[forward.index("atomicOr(status, 1)"):]
+    assert re.search(r"bar_wait\(&load_bar, 0\);\s*mma_commit\(&end_bar\);\s*bar_wait\(&end_bar, 0\);", gave_up)
+    # the parity on a model of the barrier: load n completes phase n; a wait for parity q returns at once
+    # unless the phase in progress has parity q
+    for tiles in range(1, 6):
+        for landed in (tiles - 1, tiles):  # all loads but the last, or all of them
+            xph = (tiles - 1) & 1          # flipped with every load after the first
+            returns_at_once = landed & 1 != xph
+            assert returns_at_once == (landed == tiles)
