@@ -221,29 +221,50 @@ template <class R> __device__ __forceinline__ R kinvden(const KParams& p, int si
 // split: a full FP32 codec whose sweep gathers and collides f_l - Whi_l (exact for a population
 // within a factor 2 of its rest value), so that no rounding but the store's is relative to f
 // itself (cell_collide_split).
+// Loads of populations are coherent ones: a sweep launched with programmatic overlap begins while the
+// kernel that writes what it will read is still running, and a non-coherent load (__ldg, and what the
+// compiler makes of a plain load through a const __restrict__ pointer) promises data that does not
+// change while the kernel runs.  Volatile, so that none moves above griddepcontrol.wait.
+__device__ __forceinline__ double ld_pop(const double* p) {
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ld_pop(const float* p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ unsigned short ld_pop(const unsigned short* p) {
+    unsigned short v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return v;
+}
 struct CodecF64 {
     using T = double; using R = double; static constexpr bool dev = false, split = false;
-    __device__ static R ld(const T* p) { return __ldg(p); }
+    __device__ static R ld(const T* p) { return ld_pop(p); }
     __device__ static T enc(R v) { return v; }
 };
 struct CodecF32 {
     using T = float; using R = float; static constexpr bool dev = false, split = true;
-    __device__ static R ld(const T* p) { return __ldg(p); }
+    __device__ static R ld(const T* p) { return ld_pop(p); }
     __device__ static T enc(R v) { return v; }
 };
 struct CodecF32Dev {
     using T = float; using R = float; static constexpr bool dev = true, split = false;
-    __device__ static R ld(const T* p) { return __ldg(p); }
+    __device__ static R ld(const T* p) { return ld_pop(p); }
     __device__ static T enc(R v) { return v; }
 };
 struct CodecBF16Dev {
     using T = __nv_bfloat16; using R = float; static constexpr bool dev = true, split = false;
-    __device__ static R ld(const T* p) { return __bfloat162float(__ldg(p)); }
+    __device__ static R ld(const T* p) {
+        return __bfloat162float(__ushort_as_bfloat16(ld_pop(reinterpret_cast<const unsigned short*>(p))));
+    }
     __device__ static T enc(R v) { return __float2bfloat16_rn(v); }
 };
 struct CodecF16Dev {
     using T = __half; using R = float; static constexpr bool dev = true, split = false;
-    __device__ static R ld(const T* p) { return __half2float(__ldg(p)); }
+    __device__ static R ld(const T* p) { return __half2float(__ushort_as_half(ld_pop(reinterpret_cast<const unsigned short*>(p)))); }
     __device__ static T enc(R v) { return __float2half_rn(v); }
 };
 

@@ -42,3 +42,23 @@ def test_a_network_kernel_that_gives_up_waits_for_its_copies_and_products():
             xph = (tiles - 1) & 1          # flipped with every load after the first
             returns_at_once = landed & 1 != xph
             assert returns_at_once == (landed == tiles)
+
+
+def test_sweeps_that_overlap_load_populations_coherently():
+    """A kernel launched with programmatic overlap begins before the kernel that writes its input has ended;
+    a non-coherent load is only defined for data that does not change while the kernel runs."""
+    text = source("tvlbm_kernels.cuh")
+    codecs = text[text.index("ld_pop(const double"):text.index("split_rest")]
+    assert "__ldg" not in codecs and ".nc" not in codecs
+    assert len(re.findall(r"static R ld\(const T\* p\)", codecs)) == len(re.findall(r"struct Codec\w+ \{", codecs)) == 5
+    # the others that read populations through __ldg are launched without overlap, every time
+    for name, kernels in (("tvlbm_kernels_impl.cuh", ["sweep_lanes_kernel", "row_pop_means_kernel", "reencode_kernel"]),
+                          ("tvlbm_fvlb.cu", ["fv_update64_kernel"]), ("tvlbm_mesh.cu", [])):
+        text, rest = source(name), source(name)
+        for kernel in kernels:
+            launches = re.findall(r"(\w+)\((\w+),\s*%s\b|\b%s(?:<[^;()]*?>)?(<<<)" % (kernel, kernel), text)
+            assert launches and all(l == ("launch_as", "false", "") or l[2] for l in launches), (kernel, launches)
+            rest = rest.replace(body_of(text, kernel), "")
+        # what remains are tables that the host wrote before the first launch
+        for arg in re.findall(r"__ldg\(([^()]*)", rest):
+            assert re.match(r"(src|wt|len|h|fp\.ysc) ?\+", arg), (name, arg)
