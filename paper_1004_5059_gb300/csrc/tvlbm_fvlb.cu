@@ -905,22 +905,13 @@ __global__ void __launch_bounds__(32) fv_update64_kernel(const double* __restric
     store_with_images(fout, geom_of(p), (long long)l * p.plane, x, y, out);
 }
 
-int fv_sm_count() {
-    static int n[64] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64) return 152;
-    if (!n[dev]) cudaDeviceGetAttribute(&n[dev], cudaDevAttrMultiProcessorCount, dev);
-    return n[dev] > 0 ? n[dev] : 152;
-}
-
 template <int N1, class C>
 cudaError_t launch_fv(const void* f, void* om, void* fout, const KParams& p, const FvParams& fp, const WallParams& wp,
                       bool split, cudaStream_t s) {
     using T = typename C::T;
     cudaError_t e = cudaSuccess;
     const long long gx = (p.nx + 31) / 32;
-    const int sms = fv_sm_count();
+    const int sms = sm_count();
     // FP64 runs the collision term and the update as two kernels in either form: its time is FP64
     // instructions, and the two kernels compute every collision term once (the march of the fused
     // form recomputes those of its ring)

@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <type_traits>
 #include <utility>
 
@@ -399,6 +400,20 @@ __device__ __forceinline__ void cell_collide(R (&s)[N1 * N1], const KParams& p, 
 // writes are complete and visible (wait).  Both are no-ops when launched without the attribute.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// SMs of the current device, which the lines between kernels and the splits of work count in (152,
+// GB300's, where there is no device to ask).
+inline int sm_count() {
+    static std::atomic<int> sms[64];
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 152;
+    n = sms[dev].load(std::memory_order_relaxed);
+    if (n == 0) {
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 152;
+        sms[dev].store(n, std::memory_order_relaxed);
+    }
+    return n;
+}
 
 // Launch a kernel, with programmatic stream serialization (see pdl_wait) or without.
 template <class... KArgs, class... Args>

@@ -156,14 +156,6 @@ __global__ void __launch_bounds__(32) sweep_lanes_kernel(const double* __restric
 // instead of 37), up to 600 cells per SM (256 x 256 37 against 51 to 72 us tiled; 500 x 300 79.7 against
 // 76.3), and lanes sharing a cell up to 64 cells per SM (32 for D2Q36, whose cells take 8 lanes): 64 x
 // 64 D2Q16 5.6 against 11.8 us with one lane per cell, 128 x 80 10.7 with one.
-inline int sm_count() {
-    static int sms[64] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64) return 0;
-    if (!sms[dev]) cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev);
-    return sms[dev];
-}
 template <int N1, class C>
 inline bool sweep_without_tiles(const KParams& p) {
     const long long cells = (long long)p.nx * p.ny;

@@ -62,3 +62,9 @@ def test_sweeps_that_overlap_load_populations_coherently():
         # what remains are tables that the host wrote before the first launch
         for arg in re.findall(r"__ldg\(([^()]*)", rest):
             assert re.match(r"(src|wt|len|h|fp\.ysc) ?\+", arg), (name, arg)
+
+
+def test_one_count_of_the_sms():
+    """The lines between kernels and the splits of work use one SM count, with one fallback."""
+    defined = [n for n in sorted(os.listdir(CSRC)) if re.search(r"\bint \w*sm_count\(\) \{", source(n))]
+    assert defined == ["tvlbm_kernels.cuh"]
