@@ -259,6 +259,16 @@ int tvlbm_tile_count(const tvlbm_ctx *ctx);
 int tvlbm_tile_shape(const tvlbm_ctx *ctx, int config, int *tx, int *ty, int *rows_per_thread);
 int tvlbm_set_tile(tvlbm_ctx *ctx, int config);
 
+/* Small domains run faster without tiles (one cell per thread, or lanes sharing an FP64 cell), so the
+ * tiled form runs them that way: the same populations, whatever tile configuration is selected.
+ * tvlbm_set_always_tiles(ctx, 1) keeps the tiles on every domain (0, the default, returns to the rule);
+ * tvlbm_runs_tiles says whether the context's next step runs tiles, i.e. whether the tile configuration
+ * matters (1 or 0); tvlbm_tiled_form_tiles says it for a domain of these sizes under the rule, without a
+ * context.  Errors: EINVAL (null context; sizes, set or storage that tvlbm_create refuses). */
+int tvlbm_set_always_tiles(tvlbm_ctx *ctx, int enable);
+int tvlbm_runs_tiles(const tvlbm_ctx *ctx);
+int tvlbm_tiled_form_tiles(int nx, int ny, int velset, int storage);
+
 /* Initialise every cell to the equilibrium f_eq(rho, u, T) (Sec. "The TVLBM model"),
  * computed in FP64 and rounded to the storage format.  Host FP64 fields [ny][nx];
  * requires rho > 0 and T > 0 everywhere (EINVAL otherwise, nothing written).

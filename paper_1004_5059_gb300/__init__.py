@@ -86,6 +86,9 @@ def _load_library() -> ctypes.CDLL:
         "tvlbm_tile_count": (_I, [_P]),
         "tvlbm_tile_shape": (_I, [_P, _I, _IP, _IP, _IP]),
         "tvlbm_set_tile": (_I, [_P, _I]),
+        "tvlbm_set_always_tiles": (_I, [_P, _I]),
+        "tvlbm_runs_tiles": (_I, [_P]),
+        "tvlbm_tiled_form_tiles": (_I, [_I, _I, _I, _I]),
         "tvlbm_init_moments": (_I, [_P, _DP, _DP, _DP, _DP]),
         "tvlbm_step": (_I, [_P, _I]),
         "tvlbm_moments": (_I, [_P, _DP, _DP, _DP, _DP]),
@@ -239,6 +242,20 @@ def tvlbm_tile_shape(ctx, config: int):
 
 def tvlbm_set_tile(ctx, config: int):
     _check(_lib.tvlbm_set_tile(ctx, int(config)), ctx)
+
+
+def tvlbm_set_always_tiles(ctx, enable: bool):
+    _check(_lib.tvlbm_set_always_tiles(ctx, 1 if enable else 0), ctx)
+
+
+def tvlbm_runs_tiles(ctx) -> bool:
+    return _lib.tvlbm_runs_tiles(ctx) == 1
+
+
+def tvlbm_tiled_form_tiles(nx: int, ny: int, velset: int, storage: int) -> bool:
+    rc = _lib.tvlbm_tiled_form_tiles(int(nx), int(ny), int(velset), int(storage))
+    _check(min(rc, TVLBM_OK))
+    return rc == 1
 
 
 def tvlbm_init_moments(ctx, rho, ux, uy, T):
@@ -396,6 +413,14 @@ class Simulation:
 
     def set_tile(self, config: int):
         tvlbm_set_tile(self.ctx, config)
+
+    def set_always_tiles(self, enable=True):
+        """Tiled form: tiles on small domains too, which it otherwise runs without (the same populations)."""
+        tvlbm_set_always_tiles(self.ctx, enable)
+
+    def runs_tiles(self) -> bool:
+        """Whether the next step runs tiles, i.e. whether the tile configuration matters."""
+        return tvlbm_runs_tiles(self.ctx)
 
     def set_reference(self, ux: float, uy: float, T: float):
         tvlbm_set_reference(self.ctx, ux, uy, T)

@@ -69,7 +69,8 @@ cudaError_t launch_step(tvlbm_ctx* c, int from, cudaStream_t s) {
         if (e != cudaSuccess) return e;
     }
     const SweepMaps maps = {c->form == FORM_STRIP ? &c->rmap[from] : &c->tmap[from], nullptr};
-    return c->kt->sweep(c->storage, c->form, c->tile_cfg, fin, fout, &maps, c->kp, s);
+    const int form = c->form == FORM_TILED && c->always_tiles ? FORM_TILES : c->form;
+    return c->kt->sweep(c->storage, form, c->tile_cfg, fin, fout, &maps, c->kp, s);
 }
 
 // Tile grid of configuration cfg when the dataflow form can run it: a periodic domain that the
@@ -558,6 +559,37 @@ int tvlbm_set_tile(tvlbm_ctx* c, int config) {
     }
     drop_graphs(c);
     return TVLBM_OK;
+}
+
+int tvlbm_tiled_form_tiles(int nx, int ny, int velset, int storage) {
+    char msg[256];
+    const int rc = validate(nx, ny, velset, 1.0, 1.0 / 8.0, nullptr, storage, 1.0, msg, sizeof(msg));
+    if (rc) return rc;
+    const int n = nodes_for(velset);
+    const Layout L = make_layout(nx, ny, n * n, storage);
+    KParams p;
+    memset(&p, 0, sizeof(p));
+    p.nx = nx;
+    p.ny = ny;
+    p.pitch = L.pitch;
+    p.rows = L.rows;
+    p.plane = L.plane;
+    return table_for(n)->without_tiles(storage, p) ? 0 : 1;
+}
+
+int tvlbm_set_always_tiles(tvlbm_ctx* c, int enable) {
+    if (!c) return TVLBM_EINVAL;
+    const int on = enable ? 1 : 0;
+    if (on != c->always_tiles) drop_graphs(c);
+    c->always_tiles = on;
+    return TVLBM_OK;
+}
+
+int tvlbm_runs_tiles(const tvlbm_ctx* c) {
+    if (!c) return TVLBM_EINVAL;
+    if (c->scheme != TVLBM_SCHEME_VOLUMETRIC || c->mesh_mem) return 0;
+    if (c->form == FORM_TILED) return c->always_tiles || !c->kt->without_tiles(c->storage, c->kp) ? 1 : 0;
+    return c->form == FORM_FLOW ? 1 : 0;
 }
 
 int tvlbm_init_moments(tvlbm_ctx* c, const double* rho, const double* ux, const double* uy, const double* T) {

@@ -42,6 +42,7 @@ struct tvlbm_ctx {
     cudaGraphExec_t graph[2];
     int have_tmap;
     int tile_cfg;                     // tiled-form tile configuration
+    int always_tiles;                 // tiled form: tiles on small domains too
     alignas(64) CUtensorMap tmap[2];  // TMA descriptors: input windows of buffer b
     alignas(64) CUtensorMap smap[2];  //   and one tile of buffer b (the dataflow form's TMA stores)
     alignas(64) CUtensorMap rmap[2];  //   and one source row of buffer b (the warp-strip form)

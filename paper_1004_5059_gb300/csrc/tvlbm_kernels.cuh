@@ -57,6 +57,7 @@ static_assert(kMaxQ % 4 == 0 && kRowF % 4 == 0, "row entries are read as float4"
 
 enum Storage { ST_FP64 = 0, ST_FP32 = 1, ST_BF16_DEV = 2, ST_FP16_DEV = 3, ST_FP32_DEV = 4 };
 enum Form { FORM_PLAIN = 0, FORM_TILED = 1, FORM_FLOW = 2, FORM_STRIP = 3 };
+constexpr int FORM_TILES = 256;  // FORM_TILED with tiles on every domain (tvlbm_set_tiles; sweep launches only)
 
 // Everything a kernel needs, passed by value (lands in the constant bank).
 struct KParams {
@@ -524,6 +525,8 @@ struct KernelTable {
     cudaError_t (*row_pop_means)(int storage, const void* f, double* prof, const KParams& p, cudaStream_t s);
     // per-row reference tables whose Pref is the profile prof [Q][ny] itself
     cudaError_t (*ref_tables_mean)(const double* prof, double* rowd, float* rowf, const KParams& p, cudaStream_t s);
+    // whether FORM_TILED runs the domain without tiles
+    bool (*without_tiles)(int storage, const KParams& p);
 };
 
 const KernelTable* kernel_table_q3();

@@ -618,7 +618,7 @@ struct Launch {
                                cudaStream_t s) {
         using T = typename C::T;
         const bool small = form == FORM_TILED && sweep_without_tiles<N1, C>(p);
-        if (form == FORM_TILED && !small) return tiled_sweep<N1, C>(cfg, maps, (T*)fout, p, s);
+        if (form == FORM_TILES || (form == FORM_TILED && !small)) return tiled_sweep<N1, C>(cfg, maps, (T*)fout, p, s);
         if (form == FORM_STRIP) return strip_sweep<N1, C>(maps, (T*)fout, p, s);
         constexpr bool F64 = sizeof(T) == 8;
         if constexpr (F64) {
@@ -806,11 +806,20 @@ struct Launch {
         }
     }
 #undef TVLBM_DISPATCH
+    static bool without_tiles(int storage, const KParams& p) {
+        switch (storage) {
+            case ST_FP64: return sweep_without_tiles<N1, CodecF64>(p);
+            case ST_FP32: return sweep_without_tiles<N1, CodecF32>(p);
+            case ST_BF16_DEV: return sweep_without_tiles<N1, CodecBF16Dev>(p);
+            case ST_FP16_DEV: return sweep_without_tiles<N1, CodecF16Dev>(p);
+            default: return sweep_without_tiles<N1, CodecF32Dev>(p);
+        }
+    }
 
     static const KernelTable* table() {
         static const KernelTable t = {&sweep, &init, &moments, &reduce, &wall, &halo, &decode, &encode, &tiled_available,
                                       &box, &shape, &reencode, &flow, &batch, &batch_flow, &row_means, &ref_tables,
-                                      &row_pop_means, &ref_tables_mean};
+                                      &row_pop_means, &ref_tables_mean, &without_tiles};
         return &t;
     }
 };
