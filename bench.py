@@ -348,7 +348,7 @@ def run_ours(args, w, rank, world, local_rank, sub=None):
                                                  form)
                 tr = autotune.autotune(sim, steps=min(tsteps, 100), repeats=3, log_path=log, form=form)
                 for t in tr["trials"]:
-                    trials["%s %s" % (form, tuple(t["tile"]))] = round(t["s_per_step"] * 1e6, 2)
+                    trials["%s %s" % (form, tuple(t["tile"]) if t["tile"] else "without tiles")] = round(t["s_per_step"] * 1e6, 2)
                 best_t = min(t["s_per_step"] for t in tr["trials"])
                 if tuning is not None and best_t >= tuning["s_per_step"]:
                     sim.close()
@@ -419,7 +419,7 @@ def run_ours(args, w, rank, world, local_rank, sub=None):
                   "fp32_dev": "f32"}[w["storage"]],
         "data": "synthetic (seeded fields shaped like the paper's test problems)",
         "config": {"workload": w["desc"], "nx": nx, "ny": ny, "velset": w["velset"], "storage": w["storage"],
-                   "tau": w["tau"], "time_steps_per_bench_step": tsteps, "form": chosen,
+                   "tau": w["tau"], "time_steps_per_bench_step": tsteps, "form": form_label(probe, chosen),
                    "deviation_reference": ("per row: the start's equilibria (u = 0, T linear between the walls), "
                                            "reset every %d steps inside the timed region to the rows' %s" % (
                                                w.get("refresh", 0),
@@ -477,12 +477,17 @@ def run_ours(args, w, rank, world, local_rank, sub=None):
 def form_tile(tv, sim, form, cfg):
     """The sweep's work shape: (tile width, tile height, rows per thread) of the tiled and
     dataflow forms; (128 columns, 1 row, 1 row) for the strip form, whose CTAs walk 128-column
-    strips a row at a time; None for the plain form."""
-    if form == "plain":
+    strips a row at a time; None for the plain form and where the tiled form runs without tiles."""
+    if form == "plain" or (form == "tiled" and not sim.runs_tiles()):
         return None
     if form == "strip":
         return [128, 1, 1]
     return list(tv.tvlbm_tile_shape(sim.ctx, cfg))
+
+
+def form_label(sim, form):
+    """The form as reported: the tiled form says where it runs without tiles."""
+    return form if form != "tiled" or sim.runs_tiles() else "tiled (without tiles)"
 
 
 def autotune_log_path(args):
@@ -569,7 +574,7 @@ def sub_record(name, w, sim, form, tuning, trials, timed, fields, tv, K=3, W=2):
     peak, peak_kind = measured_peak_hbm()
     achieved = bpc * nx * ny / s_per_tstep / 1e9
     rec = {"workload": w["desc"], "value": nx * ny / s_per_tstep / 1e6, "unit": UNIT, "ms_per_step": ms / K,
-           "steps": K, "warmup": W, "form": form, "storage": w["storage"],
+           "steps": K, "warmup": W, "form": form_label(sim, form), "storage": w["storage"],
            "tile": form_tile(tv, sim, form, tuning["best"]) if tuning else None,
            "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                         "peak_kind": peak_kind, "bytes_per_cell": bpc,

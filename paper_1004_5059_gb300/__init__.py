@@ -350,6 +350,7 @@ class Simulation:
         self.velset = VELSETS[velset] if isinstance(velset, str) else int(velset)
         self.storage = STORAGES[storage] if isinstance(storage, str) else int(storage)
         self.Q = self.velset
+        self._tile = 0
         bc = None if walls is None else tuple(float(v) for v in walls)
         nbytes = tvlbm_memory_bytes(self.nx, self.ny, self.velset, bc, self.storage)
         self._mem = torch.empty(nbytes + 256, dtype=torch.uint8, device="cuda")
@@ -413,6 +414,11 @@ class Simulation:
 
     def set_tile(self, config: int):
         tvlbm_set_tile(self.ctx, config)
+        self._tile = int(config)
+
+    def tile(self) -> int:
+        """The selected tile configuration."""
+        return self._tile
 
     def set_always_tiles(self, enable=True):
         """Tiled form: tiles on small domains too, which it otherwise runs without (the same populations)."""

@@ -3,10 +3,12 @@
 For one context it times every tile configuration the library offers (tvlbm_tile_count /
 tvlbm_tile_shape / tvlbm_set_tile) with CUDA events on the context's stream, keeps the fastest,
 and appends one JSON record per trial to a log -- (grid, velocity set, storage, form, tile
-shape, configuration, seconds per time step).  `predict` is the shape -> configuration model
-trained on that log: for a grid that was never tuned it returns the configuration that won on
-the nearest logged grid of the same velocity set, storage and form.  Timing runs advance the
-simulation, so tune on a scratch context (or reinitialise).
+shape, configuration, seconds per time step).  A context whose next step runs no tiles
+(tvlbm_runs_tiles: the tiled form on a small domain) has nothing to choose: one trial without a
+tile shape, not logged.  `predict` is the shape -> configuration model trained on that log: for a
+grid that was never tuned it returns the configuration that won on the nearest logged grid of the
+same velocity set, storage and form.  Timing runs advance the simulation, so tune on a scratch
+context (or reinitialise).
 """
 from __future__ import annotations
 
@@ -50,7 +52,12 @@ def default_log_path() -> str:
 
 def autotune(sim, steps: int = 64, repeats: int = 3, log_path: str | None = None, form: str | None = None) -> dict:
     """Select the fastest tile configuration for `sim` (left selected) and return the trials;
-    with `log_path`, append them to that log (`form` labels the records)."""
+    with `log_path`, append them to that log (`form` labels the records).  Where the context runs
+    no tiles, the configuration stays as it is and the one trial's "tile" is None."""
+    if not sim.runs_tiles():
+        cfg = sim.tile()
+        trials = [{"config": cfg, "tile": None, "s_per_step": time_config(sim, cfg, steps, repeats)}]
+        return {"nx": sim.nx, "ny": sim.ny, "velset": sim.velset, "storage": sim.storage, "best": cfg, "trials": trials}
     shapes = tile_shapes(sim)
     trials = []
     for cfg, shape in enumerate(shapes):
@@ -87,10 +94,19 @@ def read_log(log_path: str) -> list[dict]:
     return out
 
 
+def _tiles_matter(nx: int, ny: int, velset: int, storage: int) -> bool:
+    """Whether the tiled form runs this grid with tiles (also for sizes the library does not know)."""
+    try:
+        return tv.tvlbm_tiled_form_tiles(nx, ny, velset, storage)
+    except tv.TvlbmError:
+        return True
+
+
 def predict(records: list[dict], nx: int, ny: int, velset: int, storage: int, form: str | None = None) -> dict | None:
     """Configuration for an nx x ny grid from logged trials: per logged grid (same velocity set,
     storage and form) the configuration with the lowest median time per time step; of those
-    grids, the one nearest in (log2 cells, log2 aspect ratio).  None when nothing matches.
+    grids, the one nearest in (log2 cells, log2 aspect ratio).  Grids that the tiled form runs
+    without tiles say nothing about a tile and are left out.  None when nothing matches.
     Returns {"config", "tile", "from": [nx, ny], "distance"}."""
     per_grid: dict[tuple[int, int], dict[int, list]] = {}
     for r in records:
@@ -99,6 +115,8 @@ def predict(records: list[dict], nx: int, ny: int, velset: int, storage: int, fo
         try:
             key, cfg, t = (int(r["nx"]), int(r["ny"])), int(r["config"]), float(r["s_per_step"])
         except (KeyError, TypeError, ValueError):
+            continue
+        if form == "tiled" and not _tiles_matter(*key, velset, storage):
             continue
         per_grid.setdefault(key, {}).setdefault(cfg, [r.get("tile"), []])[1].append(t)
     best = None
