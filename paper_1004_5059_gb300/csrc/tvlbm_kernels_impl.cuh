@@ -140,17 +140,48 @@ __global__ void __launch_bounds__(32) sweep_lanes_kernel(const double* __restric
         }
 }
 
+// What the lines between the kernels count in: warps of 31 and of 32 columns in a row, the populations
+// that whole warps of 32 columns cover, the bytes of both buffers, frame included.
+template <int N1, class C>
+struct SweepSize {
+    static constexpr int ES = (int)sizeof(typename C::T);
+    long long w31, w32, covered, bytes;
+    explicit SweepSize(const KParams& p)
+        : w31((p.nx + 30) / 31), w32((p.nx + 31) / 32), covered(w32 * 32 * p.ny * (N1 * N1)),
+          bytes(2 * p.plane * (N1 * N1) * ES) {}
+};
+// The shuffled gather where its warps are more than the resident ones (below, the extra latency counts:
+// D2Q16 FP32 320 x 320 4.8 us per step against 4.2 with four loads, 384 x 384 5.1 against 5.2, 16 x 4096
+// 5.3 against 5.5), where 31 columns to a warp make at most one warp in eight more than 32 do (FP32
+// deviations, D2Q16: 224 x 2500 15.5 against 16.2, 192 x 2500 13.8 against 13.5, 64 x 4096 12.0 against
+// 9.3, 32 x 8192 15.1 against 9.6; D2Q36 in 2-byte storage up to one in three, 128 x 4096 38 against 52, 64 x
+// 2048 14.5 against 14.1), and where both buffers stay in the L2 cache (1000 x 601 D2Q16 FP32
+// 14.4 against 16.0, D2Q36 512 x 512 FP32 16.8 against 19.1): beyond it the stores of the 31-column
+// rows, which share sectors between blocks, cost memory traffic (1024 x 1024 FP32 32.7 against 30.8), unless
+// one warp has the whole row (1 x 60000 D2Q36 FP16 263 against 360).  D2Q9 has too little to load.
+template <int N1, class C>
+inline bool sweep_by_shuffle(const KParams& p) {
+    if (N1 == 3) return false;
+    const SweepSize<N1, C> z(p);
+    const bool few_more = 7 * z.w31 <= 8 * z.w32 || (N1 == 6 && z.ES == 2 && 3 * z.w31 <= 4 * z.w32);
+    return z.w31 * p.ny >= (N1 == 4 ? 4000 : 2000) && few_more && (p.nx <= 16 || z.bytes <= 130000000LL);
+}
 // The tiled form runs small domains without tiles (the same bits).  A tile's windows take a TMA round
 // trip and its threads walk 2 to 4 rows one after another, which a small grid has no other work to
 // hide: 100 x 75 D2Q9 FP32 4.9 us per step tiled against 2.5 with one cell per thread, 128 x 128
 // D2Q16 6.4 against 2.9.  The line lies where the tiles' fewer loads (each value once, not twice or four
-// times through the L1 cache) and whole-row stores begin to pay: at 15 M populations in 4-byte storage
-// (without tiles against tiled: 1000 x 601 D2Q16 FP32 15.3 against 19.0 us, 960 x 960 27.4 against 27.7,
-// 1024 x 1024 34 against 31; 640 x 600 D2Q36 29.5 against 33.6), in 2-byte storage, whose single loads carry
-// half as much, at 8 M for D2Q9 (1000 x 950 15.2 against 16.0, 1300 x 1300 25.0 against 23.6), 15 M for
-// D2Q16 (768 x 768 14.7 against 16.7, 980 x 980 22.5 against 22.7) and 30 M for D2Q36, where the tiles'
-// windows leave few warps (channels: 1024 x 512 33.6 against 38.3, 1000 x 900 57.1 against 58.7, 2048 x 512
-// 63.2 against 62.2).  FP64 is bound by its arithmetic, so what counts is an even spread over the
+// times through the L1 cache) and whole-row stores begin to pay, in populations that whole warps cover.
+// Shuffled: 15.6 M (without tiles against tiled: 1000 x 601 D2Q16 FP32 15.3 against 19.0 us, 960 x 960 26.1
+// against 27.7, 1024 x 1024 34 against 31; 640 x 600 D2Q36 29.5 against 33.6; 16 x 32768 D2Q16 FP16, half
+// its warps empty, 46.9 against 42.0), and 32 M for D2Q36 in 2-byte storage, where the tiles' windows leave few
+// warps (channels: 1024 x 512 33.6 against 38.3, 1000 x 900 57.1 against 58.7, 2048 x 512 63.2 against 62.2;
+// 19 M where the 31-column warps are over one in eight more: 128 x 4096 37 against 41, 96 x 6000 54
+// against 48); a domain of up to 8 columns, whose tiles are mostly frame, never takes them (8 x 20000 D2Q36
+// FP32 64 against 68, 1 x 60000 D2Q16 FP32 104 against 111).  With four loads: D2Q9 15.6 M, 9 M in 2-byte
+// storage (1000 x 950 15.2 against 16.0, 1300 x 1300 25.0 against 23.6, 16 x 32768 22.0 against 21.5); D2Q16 10 M
+// and buffers of 97 MB in 4-byte storage (64 x 6000 12.9 against 14.2, 32 x 12000 17.9 against 17.2), 8 M in
+// 2-byte (64 x 6000 14.1 against 17.3, 64 x 8192 18.6 against 18.0); D2Q36 7 M (FP32 64 x 2048 11.8 against 14.5, 64 x 4096 35.3
+// against 31.7).  FP64 is bound by its arithmetic, so what counts is an even spread over the
 // SM partitions: blocks of one warp, launched without programmatic overlap (blocks placed around those
 // of a kernel still resident share partitions: 64 x 64 D2Q16 8.5 instead of 5.6 us, 256 x 256 59
 // instead of 37), up to 600 cells per SM (256 x 256 37 against 51 to 72 us tiled; 500 x 300 79.7 against
@@ -158,22 +189,31 @@ __global__ void __launch_bounds__(32) sweep_lanes_kernel(const double* __restric
 // 64 D2Q16 5.6 against 11.8 us with one lane per cell, 128 x 80 10.7 with one.
 template <int N1, class C>
 inline bool sweep_without_tiles(const KParams& p) {
-    const long long cells = (long long)p.nx * p.ny;
     if (p.ny > 65535) return false;  // rows of blocks: the grid's y extent
-    if (sizeof(typename C::T) == 8) return cells <= 600LL * sm_count();
-    return cells * (N1 * N1) <= (sizeof(typename C::T) == 4 || N1 == 4 ? 15000000LL : N1 == 3 ? 8000000LL : 30000000LL);
+    const SweepSize<N1, C> z(p);
+    if (z.ES == 8) return (long long)p.nx * p.ny <= 600LL * sm_count();
+    if (N1 == 3) return z.covered <= (z.ES == 4 ? 15600000LL : 9000000LL);
+    if (sweep_by_shuffle<N1, C>(p)) {
+        if (p.nx <= 8) return true;
+        return z.covered <= (N1 == 6 && z.ES == 2 ? (7 * z.w31 <= 8 * z.w32 ? 32000000LL : 19000000LL) : 15600000LL);
+    }
+    if (N1 == 6) return z.covered <= 7000000LL;
+    return z.covered <= (z.ES == 4 ? 10000000LL : 8000000LL) && (z.ES == 2 || z.bytes <= 97000000LL);
 }
-// The shuffled gather where the cells are more than the resident warps' (below, the extra latency
-// counts: D2Q16 FP32 360 x 300 5.0 against 4.4 us with four loads, 512 x 512 7.9 against 8.2; D2Q36 FP32 200 x 150
-// 5.8 against 5.2, 256 x 256 6.3 against 7.0) and both buffers stay in the L2 cache (1000 x 601 D2Q16 FP32
-// 15.3 against 16.9, 768 x 768 FP16 14.7 against 16.0, D2Q36 512 x 512 FP32 16.8 against 19.1, 400 x 500 FP16
-// 12.6 against 15.8): beyond it the 31-column rows, whose stores share sectors between blocks, cost
-// memory traffic (1024 x 1024 FP32 32.7 against 30.8).  D2Q9 has too little to load (1000 x 601 10.3
-// either way).
+// Rows of a block of the gather with four loads: four (128 threads; 3 to 8 % faster than eight from 128 x
+// 128 to 1024 x 1024, D2Q36 channels up to 30 %), eight where that fills the chip no worse and the rows
+// above and below, which a block loads beside its own, count: D2Q9 on grids of 1.5 to 4 such blocks per SM
+// (256 x 256 FP32 3.60 against 3.78 us per step, 64 x 2048 4.07 against 4.62; 1822 x 21, 1.1 blocks per SM,
+// 3.34 against 2.50) and D2Q36 in 4-byte storage up to one per SM (64 x 500 4.57 against 5.34, 64 x 1000
+// 8.40 against 7.68).  One row in FP64 (see above).
 template <int N1, class C>
-inline bool sweep_by_shuffle(const KParams& p) {
-    const long long cells = (long long)p.nx * p.ny;
-    return cells >= (N1 == 4 ? 250000 : 64000) && 2 * cells * (N1 * N1) * (long long)sizeof(typename C::T) <= 125000000LL;
+inline int sweep_block_rows(const KParams& p) {
+    constexpr int ES = (int)sizeof(typename C::T);
+    if (p.ny > 4 * 65535) return 8;  // the grid's y extent
+    if (ES == 8) return p.ny <= 65535 ? 1 : 4;
+    const long long blocks = (long long)((p.nx + 31) / 32) * ((p.ny + 7) / 8), sms = sm_count();
+    if (N1 == 3) return 2 * blocks > 3 * sms && blocks <= 4 * sms ? 8 : 4;
+    return N1 == 6 && ES == 4 && blocks <= sms ? 8 : 4;
 }
 template <int N1>
 inline bool sweep_in_lanes(const KParams& p) {
@@ -627,15 +667,14 @@ struct Launch {
                 return launch_as(false, sweep_lanes_kernel<N1>, dim3((unsigned)((p.nx + CELLS - 1) / CELLS * p.ny)),
                                  dim3(32), 0, s, (const T*)fin, (T*)fout, p);
         }
-        // blocks of 128 threads: 3 to 8 % faster than 256 from 128 x 128 to 1024 x 1024 (D2Q36 channels
-        // up to 30 %); one warp in FP64 (see above)
-        const dim3 b(32, p.ny > 4 * 65535 ? 8 : (F64 && p.ny <= 65535) ? 1 : 4);
+        const bool shuffle = !F64 && p.ny <= 4 * 65535 && sweep_by_shuffle<N1, C>(p);
+        const dim3 b(32, shuffle ? 4 : sweep_block_rows<N1, C>(p));
         const auto launch = [&](auto kernel, int cols) {
             const dim3 grid((p.nx + cols - 1) / cols, (p.ny + b.y - 1) / b.y);
             return launch_as(!F64, kernel, grid, b, 0, s, (const T*)fin, (T*)fout, p);
         };
         if constexpr (!F64 && N1 >= 4) {
-            if (b.y == 4 && sweep_by_shuffle<N1, C>(p)) {
+            if (shuffle) {
                 if constexpr (C::dev) {
                     if (p.rowf) return launch(sweep_plain_kernel<N1, C, true, true>, 31);
                 }
