@@ -298,22 +298,22 @@ __device__ __forceinline__ R fv_kfac(const FvParams& fp, int y, int wall) {  // 
 // PN pairs per thread (a whole cell: g = 0 .. HP - 1, i = 0 .. N1 - 1; the index functions ig, gg
 // give them).  src.row(y) moves to a row, src.get(q, ...) supplies a pair's values at the column
 // and beside it, src.own(q, y) the one at the column of row y; put(y, out) takes a finished row.  Every form of the scheme runs this one function, so they give the same bits.
-template <int N1, int PN, class R, class IG, class GG, class Src, class Put>
+template <int N1, int PN, class R, bool WALLS, class IG, class GG, class Src, class Put>
 __device__ __forceinline__ void fv_march(const KParams& p, const FvParams& fp, int y0, int y1, const IG& ig, const GG& gg,
                                          Src& src, const Put& put) {
     Pair<R> own[PN];  // f_0 of the row whose output is pending
     Pair<R> pend[PN], Lp[PN];
-    const int ra = fp.walls ? max(y0 - 1, 0) : y0 - 1, rb = fp.walls ? min(y1, p.ny - 1) : y1;
+    const int ra = WALLS && fp.walls ? max(y0 - 1, 0) : y0 - 1, rb = WALLS && fp.walls ? min(y1, p.ny - 1) : y1;
     const R dt16 = fv_const<R>(fp).dt16;
 #pragma unroll
     for (int q = 0; q < PN; ++q) Lp[q] = pend[q] = bc<R>(R(0));
 #pragma unroll 1
     for (int r = ra; r <= rb; ++r) {
         src.row(r);
-        const int wu = r > ra ? fv_wall_of(p, fp, r - 1) : 0;               // the row below (its upper neighbour is r)
-        const int wl = (r + 1 < p.ny || !fp.walls) ? fv_wall_of(p, fp, r + 1) : 0;  // the row above
-        const int wo = fv_wall_of(p, fp, r);
-        const bool ysc = fp.ysc != nullptr || fp.walls;
+        const int wu = WALLS && r > ra ? fv_wall_of(p, fp, r - 1) : 0;               // the row below (its upper neighbour is r)
+        const int wl = WALLS && (r + 1 < p.ny || !fp.walls) ? fv_wall_of(p, fp, r + 1) : 0;  // the row above
+        const int wo = WALLS ? fv_wall_of(p, fp, r) : 0;
+        const bool ysc = WALLS && (fp.ysc != nullptr || fp.walls);
         R kU = dt16, kL = dt16;
         if (ysc) {
             if (r > ra) kU = fv_kfac<R>(fp, r - 1, wu);
@@ -380,7 +380,7 @@ __device__ __forceinline__ void fv_march(const KParams& p, const FvParams& fp, i
             for (int q = 0; q < PN; ++q) own[q] = src.cur(q);
         }
     }
-    if (fp.walls && y1 == p.ny) {
+    if (WALLS && fp.walls && y1 == p.ny) {
 #pragma unroll
         for (int q = 0; q < PN; ++q) pend[q] = add2(src.cur(q), pend[q]);
         put(p.ny - 1, pend);
@@ -410,16 +410,19 @@ __device__ __forceinline__ void fv_unpair(const Pair<R> (&v)[fv_hp<N1>()][N1], R
         }
 }
 
-// The collision term of every cell, with its frame images.  One warp per 32 columns and row: small
-// grids (an FP64 channel of 64 x 61 nodes) then spread over as many SM partitions as they can.
+// The collision term of every cell, with its frame images: one warp per 32 columns and row.  In FP64 a warp
+// is alone in its block, so that small grids (a channel of 64 x 61 nodes) spread over as many SM
+// partitions as they can; in FP32 four make a block, since starting a block takes about 1.1 ns, more than
+// a warp of so little work leaves (see launch_fv).
 template <int N1, class C>
-__global__ void __launch_bounds__(32) fv_omega_kernel(const typename C::T* __restrict__ f, typename C::T* __restrict__ om,
+__global__ void __launch_bounds__(128) fv_omega_kernel(const typename C::T* __restrict__ f, typename C::T* __restrict__ om,
                                                       const KParams p, const FvParams fp) {
     using R = typename C::R;
     pdl_launch_dependents();
     pdl_wait();
-    const int gx = (p.nx + 31) / 32, y = blockIdx.x / gx, x = (blockIdx.x - y * gx) * 32 + threadIdx.x;
-    if (x >= p.nx) return;
+    const int gx = (p.nx + 31) / 32, by = blockIdx.x / gx, x = (blockIdx.x - by * gx) * 32 + threadIdx.x;
+    const int y = by * blockDim.y + threadIdx.y;
+    if (x >= p.nx || y >= p.ny) return;
     Pair<R> s[fv_hp<N1>()][N1], w[fv_hp<N1>()][N1];
     fv_load_cell<N1, C>(f + sidx(p, 0, x, y), p.plane, s);
     fv_omega_cell<N1, R>(s, p, fp, w);
@@ -468,18 +471,20 @@ struct FvGlobalSrc {
 };
 
 // The update from both fields in memory: one thread per (column, pair of velocities), marching over
-// `seg` rows.
-template <int N1, class C>
-__global__ void __launch_bounds__(32) fv_update_kernel(const typename C::T* __restrict__ f,
+// `seg` rows; the warps of a block take segments one above the other.  A periodic domain has its own
+// instantiation: the tests for wall rows were a third of a row's instructions (512 x 512 D2Q9 15.5 us against 12.6),
+// and a warp away from the edges stores without looking for images (11.6).
+template <int N1, class C, bool WALLS>
+__global__ void __launch_bounds__(128) fv_update_kernel(const typename C::T* __restrict__ f,
                                                        const typename C::T* __restrict__ om,
                                                        typename C::T* __restrict__ fout, const KParams p,
                                                        const FvParams fp, int seg) {
     using R = typename C::R;
     pdl_launch_dependents();
     pdl_wait();
-    const int gx = (p.nx + 31) / 32, sy = blockIdx.x / gx, x = (blockIdx.x - sy * gx) * 32 + threadIdx.x;
-    const int y0 = sy * seg, y1 = min(y0 + seg, p.ny);
-    if (x >= p.nx) return;
+    const int gx = (p.nx + 31) / 32, by = blockIdx.x / gx, x = (blockIdx.x - by * gx) * 32 + threadIdx.x;
+    const int y0 = (by * blockDim.y + threadIdx.y) * seg, y1 = min(y0 + seg, p.ny);
+    if (x >= p.nx || y0 >= p.ny) return;
     const int g = blockIdx.y / N1, i = blockIdx.y - g * N1;
     const bool single = 2 * g == N1 - 1;
     const int la = i + N1 * g, lb = single ? la : i + N1 * (N1 - 1 - g);
@@ -487,11 +492,19 @@ __global__ void __launch_bounds__(32) fv_update_kernel(const typename C::T* __re
     FvGlobalSrc<C> src{f + sidx(p, la, x, 0), f + sidx(p, lb, x, 0), om + sidx(p, la, x, 0), om + sidx(p, lb, x, 0),
                        (long long)p.pitch, 0, !single};
     src.f0 = src.fE = src.fW = src.o0 = src.oE = src.oW = Pair<R>{R(0), R(0)};
+    typename C::T *pa = fout + sidx(p, la, x, 0), *pb = fout + sidx(p, lb, x, 0);
+    const int xw = x - (int)threadIdx.x;
+    const bool inner = xw >= FILL && xw + 31 < p.nx - FILL;  // the whole warp
     const auto put = [&](int y, const Pair<R>(&out)[1]) {
+        if (inner && (WALLS || (y >= FILL && y < p.ny - FILL))) {
+            stg(pa + (long long)y * p.pitch, C::enc(out[0].x));
+            if (!single) stg(pb + (long long)y * p.pitch, C::enc(out[0].y));
+            return;
+        }
         store_with_images(fout, geo, (long long)la * p.plane, x, y, C::enc(out[0].x));
         if (!single) store_with_images(fout, geo, (long long)lb * p.plane, x, y, C::enc(out[0].y));
     };
-    fv_march<N1, 1, R>(p, fp, y0, y1, [&](int) { return i; }, [&](int) { return g; }, src, put);
+    fv_march<N1, 1, R, WALLS>(p, fp, y0, y1, [&](int) { return i; }, [&](int) { return g; }, src, put);
 }
 
 // ---- fused form ------------------------------------------------------------------------------------
@@ -618,7 +631,7 @@ __global__ void __launch_bounds__(fv_fused_warps<N1>() * 32, fv_fused_minb<N1, C
             }
         store_collided<N1, C>(fout, geo, x, y, s);
     };
-    fv_march<N1, PN, R>(p, fp, y0, y1, [](int q) { return q % N1; }, [](int q) { return q / N1; }, src, put);
+    fv_march<N1, PN, R, true>(p, fp, y0, y1, [](int q) { return q % N1; }, [](int q) { return q / N1; }, src, put);
 }
 
 // ---- wall imposition ---------------------------------------------------------------------------------
@@ -940,16 +953,21 @@ cudaError_t launch_fv(const void* f, void* om, void* fout, const KParams& p, con
         if (fp.walls) e = launch_pdl(fv_impose_kernel<N1, C>, dim3((2 * p.nx + 31) / 32), dim3(32), 0, s, (T*)f, p, wp);
         if (e != cudaSuccess) return e;
         if (split) {
-            e = launch_pdl(fv_omega_kernel<N1, C>, dim3((unsigned)(gx * p.ny)), dim3(32), 0, s, (const T*)f, (T*)om, p, fp);
+            // four warps to a block in both kernels: one-warp blocks are paced by their starts (1024 x 1024 D2Q9 without
+            // the Prandtl term 92 us per step with them, 69 with four; 128 x 128 D2Q16 9.6 and 8.5)
+            e = launch_pdl(fv_omega_kernel<N1, C>, dim3((unsigned)(gx * ((p.ny + 3) / 4))), dim3(32, 4), 0, s, (const T*)f,
+                           (T*)om, p, fp);
             if (e != cudaSuccess) return e;
-            // rows per thread: what fills 32 one-warp CTAs per SM, up to 8 (the rows above and below a
-            // segment are taken again; D2Q9 FP32 per step, 8 rows always against this: 64 x 61 13.3 and 6.5 us,
-            // 300 x 200 16.5 and 11.9)
+            // rows per thread: what gives 32 warps per SM, up to 6 (the rows above and below a
+            // segment are taken again; D2Q9 FP32 per step, 8 rows always against this: 64 x 61 13.3 and 6.3 us,
+            // 300 x 200 12.7 and 8.3; 512 x 512 17.0 with 8, 15.7 with 6, 17.5 with 2)
             const long long pairs = fv_hp<N1>() * N1;
             int seg = (int)((gx * p.ny * pairs + 32LL * sms - 1) / (32LL * sms));
-            seg = seg < 1 ? 1 : (seg > 8 ? 8 : seg);
-            return launch_pdl(fv_update_kernel<N1, C>, dim3((unsigned)(gx * ((p.ny + seg - 1) / seg)), fv_hp<N1>() * N1),
-                              dim3(32), 0, s, (const T*)f, (const T*)om, (T*)fout, p, fp, seg);
+            seg = seg < 1 ? 1 : (seg > 6 ? 6 : seg);
+            const int segs = (p.ny + seg - 1) / seg;
+            return launch_pdl(fp.walls ? fv_update_kernel<N1, C, true> : fv_update_kernel<N1, C, false>,
+                              dim3((unsigned)(gx * ((segs + 3) / 4)), fv_hp<N1>() * N1),
+                              dim3(32, 4), 0, s, (const T*)f, (const T*)om, (T*)fout, p, fp, seg);
         }
         // rows per warp: what fills the resident warps once, up to 32 (a small grid is bound by the latency
         // of the rows a warp visits and takes one row: 60 x 20 D2Q16 6.3 us against 12.1 with four)

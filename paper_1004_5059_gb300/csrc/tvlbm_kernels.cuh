@@ -454,18 +454,20 @@ __device__ __forceinline__ long long sidx(const KParams& p, int l, int x, int y)
     return (long long)l * p.plane + (long long)(y + HY) * p.pitch + (x + p.hx);
 }
 
+// The first position of fluid coordinate x, of n, in the read frame [-FILL, n + FILL): x less as many periods
+// as fit (a division only on domains narrower than the frame).
+__device__ __forceinline__ int first_image(int x, int n) {
+    if (n < FILL) return x - n * ((x + FILL) / n);
+    return x + FILL >= n ? x - n : x;
+}
 // Store v at fluid cell (x, y) and at every periodic image of it inside the read frame
 // (x in [-FILL, nx+FILL); y likewise when periodic in y).
 template <class T>
 __device__ __forceinline__ void store_with_images(T* f, const Geom& g, long long lbase, int x, int y, T v) {
-    const int x0 = x - g.nx * ((x + FILL) / g.nx);
-    if (g.walls) {
-        for (int xx = x0; xx < g.nx + FILL; xx += g.nx) stg(f + lbase + (long long)(y + HY) * g.pitch + (xx + g.hx), v);
-    } else {
-        const int y0 = y - g.ny * ((y + FILL) / g.ny);
-        for (int yy = y0; yy < g.ny + FILL; yy += g.ny)
-            for (int xx = x0; xx < g.nx + FILL; xx += g.nx) stg(f + lbase + (long long)(yy + HY) * g.pitch + (xx + g.hx), v);
-    }
+    const int x0 = first_image(x, g.nx);
+    const int y0 = g.walls ? y : first_image(y, g.ny), y1 = g.walls ? y + 1 : g.ny + FILL;
+    for (int yy = y0; yy < y1; yy += g.ny)
+        for (int xx = x0; xx < g.nx + FILL; xx += g.nx) stg(f + lbase + (long long)(yy + HY) * g.pitch + (xx + g.hx), v);
 }
 
 // TMA descriptors (CUtensorMap) of a tiled sweep: input windows (out: reserved, may be null).
