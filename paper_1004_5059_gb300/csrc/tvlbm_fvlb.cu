@@ -509,7 +509,8 @@ __global__ void __launch_bounds__(128) fv_update_kernel(const typename C::T* __r
 
 // ---- fused form ------------------------------------------------------------------------------------
 // One kernel per step: a warp owns a strip of 30 output columns (lanes 0 and 31 hold the columns
-// beside it) and marches over a segment of rows: it loads a row's populations, computes the
+// beside it; a row of up to 32 columns is periodic within its warp: 31 x 1000 D2Q16 8.4 us per step with
+// two strips of shared-memory blocks, 13.5 with two strips here) and marches over a segment of rows: it loads a row's populations, computes the
 // collision term of its 32 cells in registers, takes the east and west neighbours' values by warp
 // shuffles and carries the row's contributions to the next rows (fv_march).  The collision term
 // never leaves the registers: Q values read and Q written per cell update, 4 shuffles per velocity
@@ -532,6 +533,9 @@ __device__ __forceinline__ Pair<float> shfl_e(Pair<float> v) {
 __device__ __forceinline__ Pair<float> shfl_w(Pair<float> v) {
     return {__shfl_up_sync(0xffffffffu, v.x, 1), __shfl_up_sync(0xffffffffu, v.y, 1)};
 }
+__device__ __forceinline__ Pair<float> shfl_from(Pair<float> v, int lane) {
+    return {__shfl_sync(0xffffffffu, v.x, lane), __shfl_sync(0xffffffffu, v.y, lane)};
+}
 
 // Row source of the fused form: the lane's cell in registers, its neighbours by shuffles.  Rows come
 // through a ring of three slots in shared memory that each lane fills for itself (asynchronous copies,
@@ -543,7 +547,7 @@ __device__ __forceinline__ Pair<float> shfl_w(Pair<float> v) {
 __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
 }
-template <int N1, class C>
+template <int N1, class C, bool WHOLE>
 struct FvStripSrc {
     using R = typename C::R;
     static constexpr bool kCarry = false;
@@ -552,6 +556,7 @@ struct FvStripSrc {
     const KParams& p;
     const FvParams& fp;
     R* ring;  // [3][Q][32], at this lane
+    int east, west;  // WHOLE: the lanes that hold the columns beside this one
     int next, last, slot;  // the row whose copy is started next, the last one; the current row's slot
     Pair<R> s[fv_hp<N1>()][N1], o[fv_hp<N1>()][N1];
     __device__ __forceinline__ void start(int sl) {
@@ -593,14 +598,15 @@ struct FvStripSrc {
                                         Pair<R>& oW) const {
         f0 = s[q / N1][q % N1];
         o0 = o[q / N1][q % N1];
-        fE = shfl_e(f0);
-        fW = shfl_w(f0);
-        oE = shfl_e(o0);
-        oW = shfl_w(o0);
+        fE = WHOLE ? shfl_from(f0, east) : shfl_e(f0);
+        fW = WHOLE ? shfl_from(f0, west) : shfl_w(f0);
+        oE = WHOLE ? shfl_from(o0, east) : shfl_e(o0);
+        oW = WHOLE ? shfl_from(o0, west) : shfl_w(o0);
     }
 };
 
-template <int N1, class C>
+// WHOLE: rows of up to 32 columns, the periodic row within the warp.
+template <int N1, class C, bool WHOLE>
 __global__ void __launch_bounds__(fv_fused_warps<N1>() * 32, fv_fused_minb<N1, C>())
     fv_fused_kernel(const typename C::T* __restrict__ f, typename C::T* __restrict__ fout, const KParams p,
                     const FvParams fp, int strips, int seg) {
@@ -612,12 +618,14 @@ __global__ void __launch_bounds__(fv_fused_warps<N1>() * 32, fv_fused_minb<N1, C
     const int strip = w % strips, y0 = (w / strips) * seg;
     if (y0 >= p.ny) return;  // whole warps
     const int y1 = min(y0 + seg, p.ny);
-    const int x = strip * 30 + lane - 1;
+    const int x = WHOLE ? lane : strip * 30 + lane - 1;
     const int xl = min(x, p.nx);  // columns beyond the frame column nx belong to no output
-    const bool mine = lane >= 1 && lane <= 30 && x < p.nx;
+    const bool mine = x < p.nx && (WHOLE || (lane >= 1 && lane <= 30));
+    const int east = lane == p.nx - 1 ? 0 : min(lane + 1, 31), west = lane == 0 ? p.nx - 1 : lane - 1;
     const Geom geo = geom_of(p);
-    __shared__ R ring[fv_fused_warps<N1>()][3 * FvStripSrc<N1, C>::SLOT];
-    FvStripSrc<N1, C> src{f + sidx(p, 0, xl, 0), p, fp, &ring[threadIdx.x >> 5][lane]};
+    using Src = FvStripSrc<N1, C, WHOLE>;
+    __shared__ R ring[fv_fused_warps<N1>()][3 * Src::SLOT];
+    Src src{f + sidx(p, 0, xl, 0), p, fp, &ring[threadIdx.x >> 5][lane], east, west};
     src.begin(fp.walls ? max(y0 - 1, 0) : y0 - 1, fp.walls ? min(y1, p.ny - 1) : y1);
     const auto put = [&](int y, const Pair<R>(&out)[PN]) {
         if (!mine) return;
@@ -971,11 +979,11 @@ cudaError_t launch_fv(const void* f, void* om, void* fout, const KParams& p, con
         }
         // rows per warp: what fills the resident warps once, up to 32 (a small grid is bound by the latency
         // of the rows a warp visits and takes one row: 60 x 20 D2Q16 6.3 us against 12.1 with four)
-        const int strips = (p.nx + 29) / 30;
+        const int strips = p.nx <= 32 ? 1 : (p.nx + 29) / 30;
         long long seg = ((long long)strips * p.ny + warps - 1) / warps;
         seg = seg < 1 ? 1 : (seg > 32 ? 32 : seg);
         const long long n = strips * ((p.ny + seg - 1) / seg);
-        return launch_pdl(fv_fused_kernel<N1, C>, dim3((unsigned)((n + W - 1) / W)), dim3(W * 32), 0, s, (const T*)f,
+        return launch_pdl(p.nx <= 32 ? fv_fused_kernel<N1, C, true> : fv_fused_kernel<N1, C, false>, dim3((unsigned)((n + W - 1) / W)), dim3(W * 32), 0, s, (const T*)f,
                           (T*)fout, p, fp, strips, (int)seg);
     }
 }
