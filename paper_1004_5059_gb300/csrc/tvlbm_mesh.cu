@@ -53,8 +53,8 @@ constexpr int mesh_sweep_minb() {  // resident CTAs of 128 threads: 7 (72 regist
     return (sizeof(typename C::R) == 4 && N1 <= 4) ? 7 : 1;
 }
 
-template <int N1, class C, int KT, class Off = unsigned, int BR = 4>
-__global__ void __launch_bounds__(32 * BR, BR == 4 ? mesh_sweep_minb<N1, C>() : 1) mesh_sweep_kernel(const typename C::T* __restrict__ fin,
+template <int N1, class C, int KT, class Off = unsigned>
+__global__ void __launch_bounds__(128, sizeof(Off) == 4 ? mesh_sweep_minb<N1, C>() : 1) mesh_sweep_kernel(const typename C::T* __restrict__ fin,
                                                          typename C::T* __restrict__ fout, const KParams p,
                                                          const MeshDev m) {
     using R = typename C::R;
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(32 * BR, BR == 4 ? mesh_sweep_minb<N1, C>() : 
     pdl_launch_dependents();
     const int lane = threadIdx.x;
     const int x = blockIdx.x * 31 + lane - 1;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    const int y = (blockIdx.z * gridDim.y + blockIdx.y) * 4 + threadIdx.y;  // (z: rows beyond the grid's y extent)
     pdl_wait();
     if (y >= p.ny) return;  // whole warps
     const Off xo = (Off)(min(x, p.nx - 1) + p.hx);
@@ -218,13 +218,15 @@ cudaError_t step_as(const void* fin, void* fout, const KParams& p, const MeshDev
         if (e != cudaSuccess) return e;
     }
     // the table's row length m.k is the longest list; shorter lists are padded to it
-    const bool wide = (unsigned long long)p.plane * sizeof(T) >> 32 != 0 || p.ny > 4 * 65535;  // (the grid's y extent)
-    const dim3 block(32, wide ? 8 : 4), grid((p.nx + 30) / 31, (p.ny + block.y - 1) / block.y);
-    const auto kernel = wide       ? mesh_sweep_kernel<N1, C, 0, unsigned long long, 8>
-                        : m.k <= 2 ? mesh_sweep_kernel<N1, C, 2>
-                        : m.k == 3 ? mesh_sweep_kernel<N1, C, 3>
-                        : m.k == 4 ? mesh_sweep_kernel<N1, C, 4>
-                                   : mesh_sweep_kernel<N1, C, 0>;
+    // (planes of 4 GB or more take 64-bit offsets)
+    const bool wide = (unsigned long long)p.plane * sizeof(T) >> 32 != 0;
+    const int rows = (p.ny + 3) / 4, gz = (rows + 65534) / 65535;
+    const dim3 block(32, 4), grid((p.nx + 30) / 31, (rows + gz - 1) / gz, gz);
+    using Wide = unsigned long long;
+    const auto kernel = m.k <= 2   ? (wide ? mesh_sweep_kernel<N1, C, 2, Wide> : mesh_sweep_kernel<N1, C, 2>)
+                        : m.k == 3 ? (wide ? mesh_sweep_kernel<N1, C, 3, Wide> : mesh_sweep_kernel<N1, C, 3>)
+                        : m.k == 4 ? (wide ? mesh_sweep_kernel<N1, C, 4, Wide> : mesh_sweep_kernel<N1, C, 4>)
+                                   : (wide ? mesh_sweep_kernel<N1, C, 0, Wide> : mesh_sweep_kernel<N1, C, 0>);
     // FP64 without programmatic overlap: blocks placed around those of a kernel still resident would
     // share the SM partitions its arithmetic is bound by
     return launch_as(sizeof(T) < 8, kernel, grid, block, 0, s, (const T*)fin, (T*)fout, p, m);
