@@ -59,22 +59,9 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return r;
 }
 constexpr float kLog2e = 1.4426950408889634f;
-__device__ __forceinline__ float erf_as(float x, float& e2) {
-    const float ax = fabsf(x);
-    const float t = rcp_approx(fmaf(0.3275911f, ax, 1.0f));
-    const float poly =
-        t * fmaf(t, fmaf(t, fmaf(t, fmaf(t, 1.061405429f, -1.453152027f), 1.421413741f), -0.284496736f), 0.254829592f);
-    e2 = ex2_approx(__fmul_rn(__fmul_rn(ax, ax), -kLog2e));
-    return copysignf(fmaf(-poly, e2, 1.0f), x);
-}
-__device__ __forceinline__ float gelu_f(float z) {
-    float e2;
-    return 0.5f * z * (1.0f + erf_as(z * 0.70710678118654752f, e2));
-}
-// The same for a pair in packed FP32, per lane the operations of erf_as in their order (a packed
-// multiply, add or fused multiply-add rounds each lane as the scalar instruction; the reciprocal,
-// the exponential, |x| and the sign stay scalar; the polynomial's sign is in its coefficients):
-// 1 + erf(x), and exp(-x^2).
+// For a pair in packed FP32 (a packed multiply, add or fused multiply-add rounds each lane as the scalar
+// instruction; the reciprocal, the exponential, |x| and the sign stay scalar; the polynomial's sign is
+// in its coefficients): 1 + erf(x), and exp(-x^2).
 __device__ __forceinline__ float2 erf2_plus1(float2 x, float2& e2) {
     const float2 ax = make_float2(fabsf(x.x), fabsf(x.y));
     const float2 d = __ffma2_rn(make_float2(0.3275911f, 0.3275911f), ax, make_float2(1.0f, 1.0f));
@@ -89,13 +76,13 @@ __device__ __forceinline__ float2 erf2_plus1(float2 x, float2& e2) {
     const float2 r = __ffma2_rn(neg_poly, e2, make_float2(1.0f, 1.0f));
     return __fadd2_rn(make_float2(1.0f, 1.0f), make_float2(copysignf(r.x, x.x), copysignf(r.y, x.y)));
 }
-// Two GELUs.  The forward epilogues and tvlbm_mlp_activation's g use it.
+// Two GELUs (inference).
 __device__ __forceinline__ float2 gelu2_f(float2 z) {
     float2 e2;
     const float2 er1 = erf2_plus1(__fmul2_rn(z, make_float2(0.70710678118654752f, 0.70710678118654752f)), e2);
     return __fmul2_rn(__fmul2_rn(make_float2(0.5f, 0.5f), z), er1);
 }
-// Two GELUs and their derivatives.
+// Two GELUs and their derivatives (training): the same g as gelu2_f's.
 __device__ __forceinline__ float2 gelu2_both(float2 z, float2& dg) {
     float2 e2;
     const float2 half = make_float2(0.5f, 0.5f);
@@ -103,27 +90,22 @@ __device__ __forceinline__ float2 gelu2_both(float2 z, float2& dg) {
     dg = __ffma2_rn(__fmul2_rn(z, make_float2(0.39894228040143268f, 0.39894228040143268f)), e2, __fmul2_rn(half, er1));
     return __fmul2_rn(__fmul2_rn(half, z), er1);
 }
-__device__ __forceinline__ float gelu_grad_f(float z) {
-    float e2;
-    const float er = erf_as(z * 0.70710678118654752f, e2);
-    return fmaf(z * 0.39894228040143268f, e2, 0.5f * (1.0f + er));
-}
+// The kernels' own functions on a caller's entries, in pairs (an odd last entry beside itself): g by the
+// forward epilogues', g' by the training epilogues'.
 __global__ void activation_kernel(const float* __restrict__ z, float* __restrict__ g, float* __restrict__ dg, int n) {
-    // pairs of entries, g in the packed form of the forward epilogues (an odd last entry alone)
     for (int i = 2 * (blockIdx.x * blockDim.x + threadIdx.x); i < n; i += 2 * gridDim.x * blockDim.x) {
-        if (i + 1 < n) {
-            if (g) {
-                const float2 r = gelu2_f(make_float2(z[i], z[i + 1]));
-                g[i] = r.x;
-                g[i + 1] = r.y;
-            }
-            if (dg) {
-                dg[i] = gelu_grad_f(z[i]);
-                dg[i + 1] = gelu_grad_f(z[i + 1]);
-            }
-        } else {
-            if (g) g[i] = gelu_f(z[i]);
-            if (dg) dg[i] = gelu_grad_f(z[i]);
+        const bool two = i + 1 < n;
+        const float2 v = make_float2(z[i], z[two ? i + 1 : i]);
+        if (g) {
+            const float2 r = gelu2_f(v);
+            g[i] = r.x;
+            if (two) g[i + 1] = r.y;
+        }
+        if (dg) {
+            float2 d;
+            gelu2_both(v, d);
+            dg[i] = d.x;
+            if (two) dg[i + 1] = d.y;
         }
     }
 }

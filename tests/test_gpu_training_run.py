@@ -65,3 +65,14 @@ def test_training_run_follows_the_bf16_network(tv, rows):
         th = (th - step).astype(np.float32).astype(np.float64)  # the parameters are FP32
     assert np.linalg.norm(grad - g) <= 8e-3 * np.linalg.norm(g)
     assert np.linalg.norm(theta - th) <= 6e-2 * np.linalg.norm(th - theta0)
+
+
+def test_activation_does_not_depend_on_the_place_in_a_pair(tv):
+    """Entries are taken in pairs: an entry first, second or alone in its pair gives the same bits."""
+    import torch
+    z = torch.linspace(-9.0, 9.0, 4097, dtype=torch.float32, device="cuda")
+    g, dg = tv.mlp_activation(z)
+    g1, dg1 = tv.mlp_activation(z[1:].clone())  # every entry in the other place, an even number of them
+    assert torch.equal(g[1:], g1) and torch.equal(dg[1:], dg1)
+    g2, dg2 = tv.mlp_activation(z[2048:2049].clone())
+    assert g2.item() == g[2048].item() and dg2.item() == dg[2048].item()

@@ -68,3 +68,12 @@ def test_one_count_of_the_sms():
     """The lines between kernels and the splits of work use one SM count, with one fallback."""
     defined = [n for n in sorted(os.listdir(CSRC)) if re.search(r"\bint \w*sm_count\(\) \{", source(n))]
     assert defined == ["tvlbm_kernels.cuh"]
+
+
+def test_activation_is_the_kernels_own():
+    """tvlbm_mlp_activation runs the functions that the network's epilogues run, and there are no others."""
+    text = source("tvlbm_mlp.cu")
+    act = body_of(text, "activation_kernel")
+    assert "gelu2_f(" in act and "gelu2_f(" in body_of(text, "mlp_fused_forward_kernel")
+    assert "gelu2_both(" in act and "gelu2_both(" in body_of(text, "mlp_train_kernel")
+    assert set(re.findall(r"\b(gelu\w*)\(", text)) == {"gelu2_f", "gelu2_both"}
