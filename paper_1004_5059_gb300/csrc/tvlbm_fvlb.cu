@@ -40,7 +40,7 @@ struct FvParams {
     int prandtl;
     int pscale;         // relaxation times divided by the local pressure: tau -> tau / p, p = rho T
     int walls;          // channel: wall nodes on the first and last rows
-    const double* ysc;  // per row the y factor of its stencil [ny] (fv_rows), or null for unit spacing
+    const double* ysc;  // per row the y factor of its stencil [ny] (see fv_march), or null for unit spacing
 };
 template <class R>
 __device__ __forceinline__ const FvConst<R>& fv_const(const FvParams& p) {
@@ -96,9 +96,6 @@ __device__ __forceinline__ Pair<double> mul2(Pair<double> a, Pair<double> b) {
 __device__ __forceinline__ Pair<float> sub2(Pair<float> a, Pair<float> b) {
     const float2 r = f2sub(make_float2(a.x, a.y), make_float2(b.x, b.y));
     return {r.x, r.y};
-}
-__device__ __forceinline__ Pair<double> sub2(Pair<double> a, Pair<double> b) {
-    return {__dadd_rn(a.x, -b.x), __dadd_rn(a.y, -b.y)};
 }
 template <class R> __device__ __forceinline__ Pair<R> bc(R v) { return {v, v}; }
 __device__ __forceinline__ float mul_(float a, float b) { return __fmul_rn(a, b); }
@@ -297,7 +294,9 @@ __device__ __forceinline__ R fv_kfac(const FvParams& fp, int y, int wall) {  // 
 // taken in turn, each once, its contributions to the rows around it carried in registers.
 // PN pairs per thread (a whole cell: g = 0 .. HP - 1, i = 0 .. N1 - 1; the index functions ig, gg
 // give them).  src.row(y) moves to a row, src.get(q, ...) supplies a pair's values at the column
-// and beside it, src.own(q, y) the one at the column of row y; put(y, out) takes a finished row.  Every form of the scheme runs this one function, so they give the same bits.
+// and beside it, src.own(q, y) the one at the column of row y; put(y, out) takes a finished row.  WALLS:
+// the domain may be a channel.  Both FP32 forms run this one function, so they give the same bits (FP64
+// runs fv_update64_kernel in either form).
 template <int N1, int PN, class R, bool WALLS, class IG, class GG, class Src, class Put>
 __device__ __forceinline__ void fv_march(const KParams& p, const FvParams& fp, int y0, int y1, const IG& ig, const GG& gg,
                                          Src& src, const Put& put) {
@@ -791,8 +790,11 @@ __global__ void __launch_bounds__(32) fv_impose_kernel(typename C::T* __restrict
 // chip has 608 partitions: a 64 x 61 channel, one cell per lane, keeps 122 of them busy.  So on small
 // grids four lanes share a cell of D2Q16, each with one y-node: the moments meet in two shuffle
 // rounds, the shared scalars are computed by all four (about 95 FP64 instructions per warp instead
-// of 215; 18.7 us against 16.1 + 10.4 us for the wall imposition and one lane per cell).  A wall row first imposes its leaving populations (as fv_impose_kernel), while the other
-// rows' warps are already computing.
+// of 215; 18.7 us against 16.1 + 10.4 us for the wall imposition and one lane per cell).  A wall row first
+// imposes its leaving populations (as fv_impose_kernel), while the other rows' warps are already computing.
+// The collision term is fv_omega_cell's with the sums in another order, so FP64 populations differ in
+// their last bits between grids of up to 64 cells per SM and larger ones (one lane per cell there: D2Q9 and D2Q36
+// on every grid).
 __device__ __forceinline__ double quad_sum(double v) {
     v += __shfl_xor_sync(0xffffffffu, v, 1);
     return v + __shfl_xor_sync(0xffffffffu, v, 2);
