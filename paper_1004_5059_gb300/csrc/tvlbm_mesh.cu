@@ -53,7 +53,8 @@ constexpr int mesh_sweep_minb() {  // resident CTAs of 128 threads: 7 (72 regist
     return (sizeof(typename C::R) == 4 && N1 <= 4) ? 7 : 1;
 }
 
-template <int N1, class C, int KT, class Off = unsigned>
+// BOTH: 32 columns to a warp, every lane combining its left column too (two loads per source row, no shuffle).
+template <int N1, class C, int KT, class Off = unsigned, bool BOTH = false>
 __global__ void __launch_bounds__(128, sizeof(Off) == 4 ? mesh_sweep_minb<N1, C>() : 1) mesh_sweep_kernel(const typename C::T* __restrict__ fin,
                                                          typename C::T* __restrict__ fout, const KParams p,
                                                          const MeshDev m) {
@@ -63,7 +64,7 @@ __global__ void __launch_bounds__(128, sizeof(Off) == 4 ? mesh_sweep_minb<N1, C>
     constexpr bool PACK = std::is_same<R, float>::value && (N1 & 1) == 0 && KT > 0;
     pdl_launch_dependents();
     const int lane = threadIdx.x;
-    const int x = blockIdx.x * 31 + lane - 1;
+    const int x = BOTH ? (int)(blockIdx.x * 32) + lane : (int)(blockIdx.x * 31) + lane - 1;
     const int y = (blockIdx.z * gridDim.y + blockIdx.y) * 4 + threadIdx.y;  // (z: rows beyond the grid's y extent)
     pdl_wait();
     if (y >= p.ny) return;  // whole warps
@@ -87,16 +88,22 @@ __global__ void __launch_bounds__(128, sizeof(Off) == 4 ? mesh_sweep_minb<N1, C>
             for (int i = 0; i < H; ++i) {
                 const int mi = N1 - 1 - i, l = i + N1 * j, lm = mi + N1 * j;
                 const T *ca = fin + ((long long)l * p.plane - p.sh[i]), *cb = fin + ((long long)lm * p.plane - p.sh[mi]);
-                float2 v[KT];
+                const auto along_y = [&](const T* ca, const T* cb) {  // a source column's rows combined
+                    float2 v[KT];
 #pragma unroll
-                for (int k = 0; k < KT; ++k)
-                    v[k] = make_float2(split_rest<C>(p, l, ld_at<C, Off>(ca, ro[k])), split_rest<C>(p, lm, ld_at<C, Off>(cb, ro[k])));
-                // the first entry, then the others as lerps towards theirs (weights summing to
-                // one: a state uniform in space stays exactly uniform)
-                float2 acc = v[0];
+                    for (int k = 0; k < KT; ++k)
+                        v[k] = make_float2(split_rest<C>(p, l, ld_at<C, Off>(ca, ro[k])), split_rest<C>(p, lm, ld_at<C, Off>(cb, ro[k])));
+                    // the first entry, then the others as lerps towards theirs (weights summing to
+                    // one: a state uniform in space stays exactly uniform)
+                    float2 acc = v[0];
 #pragma unroll
-                for (int k = 1; k < KT; ++k) acc = __ffma2_rn(make_float2(ws[k], ws[k]), f2sub(v[k], v[0]), acc);
-                const float2 left = make_float2(__shfl_up_sync(0xffffffffu, acc.x, 1), __shfl_up_sync(0xffffffffu, acc.y, 1));
+                    for (int k = 1; k < KT; ++k) acc = __ffma2_rn(make_float2(ws[k], ws[k]), f2sub(v[k], v[0]), acc);
+                    return acc;
+                };
+                const float2 acc = along_y(ca, cb);
+                float2 left;
+                if constexpr (BOTH) left = along_y(ca - 1, cb - 1);
+                else left = make_float2(__shfl_up_sync(0xffffffffu, acc.x, 1), __shfl_up_sync(0xffffffffu, acc.y, 1));
                 const float2 o = __ffma2_rn(make_float2(ka<R>(p, i), ka<R>(p, mi)), f2sub(left, acc), acc);
                 s[l] = o.x;
                 s[lm] = o.y;
@@ -106,25 +113,31 @@ __global__ void __launch_bounds__(128, sizeof(Off) == 4 ? mesh_sweep_minb<N1, C>
             for (int i = 0; i < N1; ++i) {
                 const int l = i + N1 * j;
                 const T* col = fin + ((long long)l * p.plane - p.sh[i]);
-                const R v0 = split_rest<C>(p, l, ld_at<C, Off>(col, ro[0]));
-                R acc = v0;
-                if constexpr (KT > 0) {
+                const auto along_y = [&](const T* col) {
+                    const R v0 = split_rest<C>(p, l, ld_at<C, Off>(col, ro[0]));
+                    R acc = v0;
+                    if constexpr (KT > 0) {
 #pragma unroll
-                    for (int k = 1; k < KT; ++k) acc = fma(ws[k], split_rest<C>(p, l, ld_at<C, Off>(col, ro[k])) - v0, acc);
-                } else {
-                    for (int k = 1; k < m.k; ++k) {
-                        const R wk = __ldg(wt + k);
-                        if (wk == R(0)) break;  // the row's list has ended (the same row for the whole warp)
-                        const Off rk = ((Off)(__ldg(src + k) + HY) * (Off)p.pitch + xo) * (Off)sizeof(T);
-                        acc = fma(wk, split_rest<C>(p, l, ld_at<C, Off>(col, rk)) - v0, acc);
+                        for (int k = 1; k < KT; ++k) acc = fma(ws[k], split_rest<C>(p, l, ld_at<C, Off>(col, ro[k])) - v0, acc);
+                    } else {
+                        for (int k = 1; k < m.k; ++k) {
+                            const R wk = __ldg(wt + k);
+                            if (wk == R(0)) break;  // the row's list has ended (the same row for the whole warp)
+                            const Off rk = ((Off)(__ldg(src + k) + HY) * (Off)p.pitch + xo) * (Off)sizeof(T);
+                            acc = fma(wk, split_rest<C>(p, l, ld_at<C, Off>(col, rk)) - v0, acc);
+                        }
                     }
-                }
-                const R left = __shfl_up_sync(0xffffffffu, acc, 1);
+                    return acc;
+                };
+                const R acc = along_y(col);
+                R left;
+                if constexpr (BOTH) left = along_y(col - 1);
+                else left = __shfl_up_sync(0xffffffffu, acc, 1);
                 s[l] = fma(ka<R>(p, i), left - acc, acc);
             }
         }
     }
-    if (lane == 0 || x >= p.nx) return;
+    if ((lane == 0 && !BOTH) || x >= p.nx) return;
     const Geom g = geom_of(p);
     collide_cell<N1, C, false>(s, p, g, y);
     store_collided<N1, C>(fout, g, x, y, s);
@@ -221,12 +234,23 @@ cudaError_t step_as(const void* fin, void* fout, const KParams& p, const MeshDev
     // (planes of 4 GB or more take 64-bit offsets)
     const bool wide = (unsigned long long)p.plane * sizeof(T) >> 32 != 0;
     const int rows = (p.ny + 3) / 4, gz = (rows + 65534) / 65535;
-    const dim3 block(32, 4), grid((p.nx + 30) / 31, (rows + gz - 1) / gz, gz);
+    // 32 columns to a warp where 31 make too many more warps: over 1.25 times as many in FP32 D2Q9, 1.4 in FP64,
+    // 1.5 in FP32 D2Q16 and D2Q36, whose packed pairs gain most by the shuffle.  us per step, 31 against 32: FP32
+    // deviations, D2Q9 32 x 4096 7.4 and 5.2, 64 x 8192 18.0 and 13.9, 96 x 4096 12.2 and 10.6; D2Q16 32 x 4096 9.9 and
+    // 7.0; FP64 D2Q16 32 x 4096 138 and 86, 64 x 4096 205 and 170, 96 x 1024 72 and 75
+    const long long w31 = (p.nx + 30) / 31, w32 = (p.nx + 31) / 32;
+    const int most = sizeof(T) == 8 ? 28 : N1 == 3 ? 25 : 30;  // twentieths
+    const bool both = !wide && 20 * w31 > most * w32;
+    const int cols = both ? 32 : 31;
+    const dim3 block(32, 4), grid((p.nx + cols - 1) / cols, (rows + gz - 1) / gz, gz);
+    using Narrow = unsigned;
     using Wide = unsigned long long;
-    const auto kernel = m.k <= 2   ? (wide ? mesh_sweep_kernel<N1, C, 2, Wide> : mesh_sweep_kernel<N1, C, 2>)
-                        : m.k == 3 ? (wide ? mesh_sweep_kernel<N1, C, 3, Wide> : mesh_sweep_kernel<N1, C, 3>)
-                        : m.k == 4 ? (wide ? mesh_sweep_kernel<N1, C, 4, Wide> : mesh_sweep_kernel<N1, C, 4>)
-                                   : (wide ? mesh_sweep_kernel<N1, C, 0, Wide> : mesh_sweep_kernel<N1, C, 0>);
+    const auto pick = [&](auto plain, auto left_too, auto far) { return wide ? far : both ? left_too : plain; };
+    const auto kernel =
+        m.k <= 2   ? pick(mesh_sweep_kernel<N1, C, 2>, mesh_sweep_kernel<N1, C, 2, Narrow, true>, mesh_sweep_kernel<N1, C, 2, Wide>)
+        : m.k == 3 ? pick(mesh_sweep_kernel<N1, C, 3>, mesh_sweep_kernel<N1, C, 3, Narrow, true>, mesh_sweep_kernel<N1, C, 3, Wide>)
+        : m.k == 4 ? pick(mesh_sweep_kernel<N1, C, 4>, mesh_sweep_kernel<N1, C, 4, Narrow, true>, mesh_sweep_kernel<N1, C, 4, Wide>)
+                   : pick(mesh_sweep_kernel<N1, C, 0>, mesh_sweep_kernel<N1, C, 0, Narrow, true>, mesh_sweep_kernel<N1, C, 0, Wide>);
     // FP64 without programmatic overlap: blocks placed around those of a kernel still resident would
     // share the SM partitions its arithmetic is bound by
     return launch_as(sizeof(T) < 8, kernel, grid, block, 0, s, (const T*)fin, (T*)fout, p, m);

@@ -55,3 +55,18 @@ def test_taller_than_the_grid(tv, storage, heights):  # noqa: F811
     for k in range(30):
         part = out[1][:, 9000 * k:9000 * (k + 1)]
         assert np.max(np.abs(part - out[0])) <= tol * np.max(np.abs(out[0])), k
+
+
+# widths at which 32 columns to a warp, each lane combining both of its columns, take the place of 31
+@pytest.mark.parametrize("velset,storage,tol", [("D2Q9", "fp64", 1e-12), ("D2Q16", "fp64", 1e-12), ("D2Q36", "fp64", 1e-12),
+                                                ("D2Q9", "fp32", 10 * 4 * 6e-8), ("D2Q9", "fp32_dev", 10 * 4 * 6e-8)])
+@pytest.mark.parametrize("entries", [2, 3, 4, 8])
+def test_both_columns_by_one_lane(tv, velset, storage, tol, entries):  # noqa: F811
+    for nx in (31, 32, 33, 64, 65, 96):
+        sim, ref = pair(tv, nx, MESHES[entries], velset, storage, WALLS if nx % 2 else None)
+        sim.step(10)
+        ref.step(10)
+        got = sim.populations_f64()
+        err = np.max(np.abs(got - ref.f), axis=(1, 2)) / np.max(np.abs(ref.f), axis=(1, 2))
+        assert np.max(err) <= tol, (nx, err)
+        sim.close()
