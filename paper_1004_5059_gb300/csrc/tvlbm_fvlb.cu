@@ -487,7 +487,8 @@ __global__ void __launch_bounds__(128) fv_update_kernel(const typename C::T* __r
     const int g = blockIdx.y / N1, i = blockIdx.y - g * N1;
     const bool single = 2 * g == N1 - 1;
     const int la = i + N1 * g, lb = single ? la : i + N1 * (N1 - 1 - g);
-    const Geom geo = geom_of(p);
+    Geom geo = geom_of(p);
+    geo.walls = WALLS;
     FvGlobalSrc<C> src{f + sidx(p, la, x, 0), f + sidx(p, lb, x, 0), om + sidx(p, la, x, 0), om + sidx(p, lb, x, 0),
                        (long long)p.pitch, 0, !single};
     src.f0 = src.fE = src.fW = src.o0 = src.oE = src.oW = Pair<R>{R(0), R(0)};
@@ -773,7 +774,8 @@ __global__ void __launch_bounds__(32) fv_impose_kernel(typename C::T* __restrict
     }
     WallFactors<N1> wf;
     wf.set(wp, ue, Te, inc);
-    const Geom g = geom_of(p);
+    Geom g = geom_of(p);
+    g.walls = 1;
 #pragma unroll
     for (int jj = 0; jj < H; ++jj) {
         const int j = side == 0 ? N1 - 1 - jj : jj;  // c . n > 0

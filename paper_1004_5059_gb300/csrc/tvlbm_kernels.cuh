@@ -465,9 +465,12 @@ __device__ __forceinline__ int first_image(int x, int n) {
 template <class T>
 __device__ __forceinline__ void store_with_images(T* f, const Geom& g, long long lbase, int x, int y, T v) {
     const int x0 = first_image(x, g.nx);
-    const int y0 = g.walls ? y : first_image(y, g.ny), y1 = g.walls ? y + 1 : g.ny + FILL;
-    for (int yy = y0; yy < y1; yy += g.ny)
-        for (int xx = x0; xx < g.nx + FILL; xx += g.nx) stg(f + lbase + (long long)(yy + HY) * g.pitch + (xx + g.hx), v);
+    if (g.walls) {
+        for (int xx = x0; xx < g.nx + FILL; xx += g.nx) stg(f + lbase + (long long)(y + HY) * g.pitch + (xx + g.hx), v);
+    } else {
+        for (int yy = first_image(y, g.ny); yy < g.ny + FILL; yy += g.ny)
+            for (int xx = x0; xx < g.nx + FILL; xx += g.nx) stg(f + lbase + (long long)(yy + HY) * g.pitch + (xx + g.hx), v);
+    }
 }
 
 // TMA descriptors (CUtensorMap) of a tiled sweep: input windows (out: reserved, may be null).
