@@ -962,7 +962,20 @@ cudaError_t launch_fv(const void* f, void* om, void* fout, const KParams& p, con
     } else {
         constexpr int W = fv_fused_warps<N1>();
         const long long warps = (long long)W * fv_fused_minb<N1, C>() * sms;  // resident warps of the fused form
-        if (fp.walls) e = launch_pdl(fv_impose_kernel<N1, C>, dim3((2 * p.nx + 31) / 32), dim3(32), 0, s, (T*)f, p, wp);
+        const int strips = p.nx <= 32 ? 1 : (p.nx + 29) / 30;
+        if (fp.walls) {
+            // The imposition is FP64: its blocks, launched early, are placed around those of the step before and share
+            // SM partitions, so it overlaps where it has few blocks and that step leaves the chip room.  us per step
+            // overlapping and not, fused: D2Q16 16 x 200 22.7 and 24.8, 256 x 200 24.4 and 27.0, 1000 x 100 27.0 and
+            // 29.0, 500 x 500 32.2 and 33.5; D2Q9 500 x 1000 50 and 39; D2Q16 2000 x 30 31 and 27, 8192 x 32 106 and 35, 1024 x
+            // 1024 139 and 69; D2Q36 256 x 200 37.6 and 39.3, 1000 x 30 37.0 and 39.2, 128 x 4000 103 and 95, 500 x 500 74 and
+            // 58.  Two kernels, whose blocks are more: D2Q16 64 x 64 20.9 and 22.8, 64 x 4000 43.1 and 45.3, 128 x 16
+            // 20.8 and 22.6, 100 x 200 24.6 and 24.0, 256 x 200 30.3 and 27.0, 500 x 16 33.1 and 22.9
+            const int blocks = (2 * p.nx + 31) / 32;
+            const bool room = 2 * blocks <= sms && (long long)blocks * strips * p.ny <= (N1 < 6 ? 300000 : 65000);
+            const bool few = blocks <= 4 || (blocks <= 8 && p.ny <= 64);
+            e = launch_as(split ? few : room, fv_impose_kernel<N1, C>, dim3(blocks), dim3(32), 0, s, (T*)f, p, wp);
+        }
         if (e != cudaSuccess) return e;
         if (split) {
             // four warps to a block in both kernels: one-warp blocks are paced by their starts (1024 x 1024 D2Q9 without
@@ -983,7 +996,6 @@ cudaError_t launch_fv(const void* f, void* om, void* fout, const KParams& p, con
         }
         // rows per warp: what fills the resident warps once, up to 32 (a small grid is bound by the latency
         // of the rows a warp visits and takes one row: 60 x 20 D2Q16 6.3 us against 12.1 with four)
-        const int strips = p.nx <= 32 ? 1 : (p.nx + 29) / 30;
         long long seg = ((long long)strips * p.ny + warps - 1) / warps;
         seg = seg < 1 ? 1 : (seg > 32 ? 32 : seg);
         const long long n = strips * ((p.ny + seg - 1) / seg);
