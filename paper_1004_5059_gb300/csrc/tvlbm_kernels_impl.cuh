@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(SHUFFLE ? 128 : 256, sweep_plain_minb<N1, SHUF
 // FP64 on a small grid: a cell shared by LG lanes (4 for D2Q9 and D2Q16, 8 for D2Q36), lane j taking the
 // populations of y-node j.  An FP64 warp instruction takes 64 cycles of its SM partition whatever its
 // active lanes, and the chip has 608 partitions; one cell per lane would leave most of them idle
-// (64 x 64 cells: 128 warps of 245 instructions, 14.6 us per step; here 512 of about 105).  The row
+// (64 x 64 cells: 128 warps of 245 instructions, 10.5 us per step; here 512 of about 105, 5.6 us).  The row
 // sums meet by shuffles, the shared factors are computed by every lane.  The arithmetic is
 // collide_cell's, piece by piece: the same bits as the other forms.
 template <int N1>
@@ -141,43 +141,51 @@ __global__ void __launch_bounds__(32) sweep_lanes_kernel(const double* __restric
 }
 
 // What the lines between the kernels count in: warps of 31 and of 32 columns in a row, the populations
-// that whole warps of 32 columns cover, the bytes of both buffers, frame included.
+// and those that whole warps of 32 columns cover, the bytes of both buffers, frame included.
 template <int N1, class C>
 struct SweepSize {
     static constexpr int ES = (int)sizeof(typename C::T);
-    long long w31, w32, covered, bytes;
+    long long w31, w32, pops, covered, bytes;
     explicit SweepSize(const KParams& p)
-        : w31((p.nx + 30) / 31), w32((p.nx + 31) / 32), covered(w32 * 32 * p.ny * (N1 * N1)),
-          bytes(2 * p.plane * (N1 * N1) * ES) {}
+        : w31((p.nx + 30) / 31), w32((p.nx + 31) / 32), pops((long long)p.nx * p.ny * (N1 * N1)),
+          covered(w32 * 32 * p.ny * (N1 * N1)), bytes(2 * p.plane * (N1 * N1) * ES) {}
 };
 // The shuffled gather where its warps are more than the resident ones (below, the extra latency counts:
 // D2Q16 FP32 320 x 320 4.8 us per step against 4.2 with four loads, 384 x 384 5.1 against 5.2, 16 x 4096
-// 5.3 against 5.5), where 31 columns to a warp make at most one warp in eight more than 32 do (FP32
-// deviations, D2Q16: 224 x 2500 15.5 against 16.2, 192 x 2500 13.8 against 13.5, 64 x 4096 12.0 against
-// 9.3, 32 x 8192 15.1 against 9.6; D2Q36 in 2-byte storage up to one in three, 128 x 4096 38 against 52, 64 x
-// 2048 14.5 against 14.1), and where both buffers stay in the L2 cache (1000 x 601 D2Q16 FP32
-// 14.4 against 16.0, D2Q36 512 x 512 FP32 16.8 against 19.1): beyond it the stores of the 31-column
-// rows, which share sectors between blocks, cost memory traffic (1024 x 1024 FP32 32.7 against 30.8), unless
-// one warp has the whole row (1 x 60000 D2Q36 FP16 263 against 360).  D2Q9 has too little to load.
+// 5.3 against 5.5; rows of up to 8 columns fill their warps less, 1 x 4096 channel 11.0 against 10.5), where
+// 31 columns to a warp make at most one warp in eight more than 32 do (FP32 deviations, D2Q16: 224 x 2500
+// 15.5 against 16.2, 192 x 2500 13.8 against 13.5, 64 x 4096 12.0 against 9.3, 32 x 8192 15.1 against 9.6;
+// D2Q36 in 2-byte storage up to one in three, 128 x 4096 38 against 52, 64 x 2048 14.5 against 14.1, and up to twice
+// as many where the buffers pass 100 MB, 64 x 8192 59 against 67, 32 x 20000 88 against 97), and where both
+// buffers stay in the L2 cache (1000 x 601 D2Q16 FP32 14.4 against 16.0, D2Q36 512 x 512 FP32 16.8 against 19.1):
+// beyond it the stores of the 31-column rows, which share sectors between blocks, cost memory traffic (1024 x
+// 1024 FP32 32.7 against 30.8), unless one warp has the whole row (1 x 60000 D2Q36 FP16 263 against 360).  D2Q36
+// loads so much that its line lies at 200 MB (FP32 48 x 8192, 151 MB, 59.0 against 65.6; FP16 960 x 960, 138 MB, 50
+// against 82).  D2Q9 has too little to load.
 template <int N1, class C>
 inline bool sweep_by_shuffle(const KParams& p) {
     if (N1 == 3) return false;
     const SweepSize<N1, C> z(p);
-    const bool few_more = 7 * z.w31 <= 8 * z.w32 || (N1 == 6 && z.ES == 2 && 3 * z.w31 <= 4 * z.w32);
-    return z.w31 * p.ny >= (N1 == 4 ? 4000 : 2000) && few_more && (p.nx <= 16 || z.bytes <= 130000000LL);
+    const bool half = N1 == 6 && z.ES == 2;
+    const bool few_more = 7 * z.w31 <= 8 * z.w32 || (half && (3 * z.w31 <= 4 * z.w32 || z.bytes > 100000000LL));
+    return z.w31 * p.ny >= (N1 == 6 ? 2000 : p.nx <= 8 ? 8000 : 4000) && few_more &&
+           (p.nx <= 16 || z.bytes <= (N1 == 6 ? 200000000LL : 130000000LL));
 }
 // The tiled form runs small domains without tiles (the same bits).  A tile's windows take a TMA round
 // trip and its threads walk 2 to 4 rows one after another, which a small grid has no other work to
 // hide: 100 x 75 D2Q9 FP32 4.9 us per step tiled against 2.5 with one cell per thread, 128 x 128
 // D2Q16 6.4 against 2.9.  The line lies where the tiles' fewer loads (each value once, not twice or four
-// times through the L1 cache) and whole-row stores begin to pay, in populations that whole warps cover.
-// Shuffled: 15.6 M (without tiles against tiled: 1000 x 601 D2Q16 FP32 15.3 against 19.0 us, 960 x 960 26.1
-// against 27.7, 1024 x 1024 34 against 31; 640 x 600 D2Q36 29.5 against 33.6; 16 x 32768 D2Q16 FP16, half
-// its warps empty, 46.9 against 42.0), and 32 M for D2Q36 in 2-byte storage, where the tiles' windows leave few
-// warps (channels: 1024 x 512 33.6 against 38.3, 1000 x 900 57.1 against 58.7, 2048 x 512 63.2 against 62.2;
-// 19 M where the 31-column warps are over one in eight more: 128 x 4096 37 against 41, 96 x 6000 54
-// against 48); a domain of up to 8 columns, whose tiles are mostly frame, never takes them (8 x 20000 D2Q36
-// FP32 64 against 68, 1 x 60000 D2Q16 FP32 104 against 111).  With four loads: D2Q9 15.6 M, 9 M in 2-byte
+// times through the L1 cache) and whole-row stores begin to pay.
+// Shuffled, in 4-byte storage: 15.6 M populations (without tiles against tiled: 1000 x 601 D2Q16 FP32 15.3
+// against 19.0 us, 960 x 960 26.1 against 27.7, 1024 x 1024 34 against 31, 16 x 32768 44.6 against 45.7; D2Q36
+// 640 x 600 29.5 against 33.6, 48 x 8192 59 against 65), for D2Q36 rows of one tile no buffers past 130 MB
+// (31 x 8192 45 against 42).  In 2-byte storage, whose tiles have whole warps, the populations these cover: 15.6
+// M for D2Q16 (16 x 32768, half its warps empty, 46.9 against 42.0) and 32 M for D2Q36, where the tiles' windows
+// leave few warps (channels: 1024 x 512 33.6 against 38.3, 1000 x 900 57.1 against 58.7, 2048 x 512 63.2 against
+// 62.2; 19 M where the 31-column warps are over one in eight more: 128 x 4096 37 against 41, 96 x 6000 54 against
+// 48; 7 M over one in three: 64 x 8192 59 against 54); a domain of up to 8 columns, whose tiles are mostly frame,
+// never takes them (8 x 20000 D2Q36 FP32 64 against 68, 1 x 60000 D2Q16 FP32 104 against 111).
+// With four loads, covered: D2Q9 15.6 M, 9 M in 2-byte
 // storage (1000 x 950 15.2 against 16.0, 1300 x 1300 25.0 against 23.6, 16 x 32768 22.0 against 21.5); D2Q16 10 M
 // and buffers of 97 MB in 4-byte storage (64 x 6000 12.9 against 14.2, 32 x 12000 17.9 against 17.2), 8 M in
 // 2-byte (64 x 6000 14.1 against 17.3, 64 x 8192 18.6 against 18.0); D2Q36 7 M (FP32 64 x 2048 11.8 against 14.5, 64 x 4096 35.3
@@ -186,7 +194,7 @@ inline bool sweep_by_shuffle(const KParams& p) {
 // of a kernel still resident share partitions: 64 x 64 D2Q16 8.5 instead of 5.6 us, 256 x 256 59
 // instead of 37), up to 600 cells per SM (256 x 256 37 against 51 to 72 us tiled; 500 x 300 79.7 against
 // 76.3), and lanes sharing a cell up to 64 cells per SM (32 for D2Q36, whose cells take 8 lanes): 64 x
-// 64 D2Q16 5.6 against 11.8 us with one lane per cell, 128 x 80 10.7 with one.
+// 64 D2Q16 5.6 against 10.5 us with one lane per cell.
 template <int N1, class C>
 inline bool sweep_without_tiles(const KParams& p) {
     if (p.ny > 65535) return false;  // rows of blocks: the grid's y extent
@@ -195,7 +203,9 @@ inline bool sweep_without_tiles(const KParams& p) {
     if (N1 == 3) return z.covered <= (z.ES == 4 ? 15600000LL : 9000000LL);
     if (sweep_by_shuffle<N1, C>(p)) {
         if (p.nx <= 8) return true;
-        return z.covered <= (N1 == 6 && z.ES == 2 ? (7 * z.w31 <= 8 * z.w32 ? 32000000LL : 19000000LL) : 15600000LL);
+        if (z.ES == 4) return z.pops <= 15600000LL && !(N1 == 6 && z.w32 == 1 && z.bytes > 130000000LL);
+        if (N1 == 4) return z.covered <= 15600000LL;
+        return z.covered <= (7 * z.w31 <= 8 * z.w32 ? 32000000LL : 3 * z.w31 <= 4 * z.w32 ? 19000000LL : 7000000LL);
     }
     if (N1 == 6) return z.covered <= 7000000LL;
     return z.covered <= (z.ES == 4 ? 10000000LL : 8000000LL) && (z.ES == 2 || z.bytes <= 97000000LL);
@@ -204,8 +214,8 @@ inline bool sweep_without_tiles(const KParams& p) {
 // 128 to 1024 x 1024, D2Q36 channels up to 30 %), eight where that fills the chip no worse and the rows
 // above and below, which a block loads beside its own, count: D2Q9 on grids of 1.5 to 4 such blocks per SM
 // (256 x 256 FP32 3.60 against 3.78 us per step, 64 x 2048 4.07 against 4.62; 1822 x 21, 1.1 blocks per SM,
-// 3.34 against 2.50) and D2Q36 in 4-byte storage up to one per SM (64 x 500 4.57 against 5.34, 64 x 1000
-// 8.40 against 7.68).  One row in FP64 (see above).
+// 3.34 against 2.50) and D2Q36 in 4-byte storage from 0.4 to one per SM (64 x 500 4.57 against 5.34, 64 x 1000
+// 8.40 against 7.68; 64 x 64, whose SMs have a block or none, 4.85 against 3.95).  One row in FP64 (see above).
 template <int N1, class C>
 inline int sweep_block_rows(const KParams& p) {
     constexpr int ES = (int)sizeof(typename C::T);
@@ -213,7 +223,7 @@ inline int sweep_block_rows(const KParams& p) {
     if (ES == 8) return p.ny <= 65535 ? 1 : 4;
     const long long blocks = (long long)((p.nx + 31) / 32) * ((p.ny + 7) / 8), sms = sm_count();
     if (N1 == 3) return 2 * blocks > 3 * sms && blocks <= 4 * sms ? 8 : 4;
-    return N1 == 6 && ES == 4 && blocks <= sms ? 8 : 4;
+    return N1 == 6 && ES == 4 && 5 * blocks >= 2 * sms && blocks <= sms ? 8 : 4;
 }
 template <int N1>
 inline bool sweep_in_lanes(const KParams& p) {
