@@ -1,4 +1,4 @@
-"""Finite-volume rows of up to 32 columns (the periodic row within a warp) and the blocks of the two-kernel
+"""Finite-volume rows of a few columns (of 31 and 32: the periodic row within a warp) and the blocks of the two-kernel
 form: the fused and the two-kernel form give the same populations bit for bit, and those of the oracle."""
 import numpy as np
 import pytest
